@@ -11,6 +11,7 @@
 //   Sec. 2.4 pose parameterisation and differentiation w.r.t. the pose
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
@@ -68,6 +69,22 @@ __device__ __forceinline__ float gather(const VolumeDev& vd, int off) {
   }
 #endif
   return Voxel<DT>::load(vd.data, off);
+}
+
+// The voxel d elements after offset off: base_d is the volume's base moved by d
+// elements (kept in registers, so the second gather of a pair costs no offset
+// addition).
+template <int DT>
+__device__ __forceinline__ float gather_at(const VolumeDev& vd, const void* base_d, int off, int d) {
+#if DRR_CHECK_BOUNDS
+  return gather<DT>(vd, off + d);
+#else
+  return Voxel<DT>::load(base_d, off);
+#endif
+}
+template <int DT>
+__device__ __forceinline__ const void* base_after(const VolumeDev& vd, int d) {
+  return static_cast<const char*>(vd.data) + static_cast<int64_t>(d) * (DT == kF32 ? 4 : 2);
 }
 
 // x_a for a runtime axis index without indexing a register array (which
@@ -274,7 +291,6 @@ __global__ void ray_setup_kernel(const float* __restrict__ poses, int B, DetDev 
 struct RayResult {
   float F;     // E (or the raw sum in alpha units before the final scaling)
   float J[6];  // dE/d eta (only for the Jacobian modes)
-  int nseg;    // number of segments (0 for a miss)
 };
 
 // Per-ray state after the FP64 setup: everything the walk needs.
@@ -328,18 +344,20 @@ __device__ __forceinline__ int floor_fast(double x) {
   return static_cast<int>(floor(x));
 }
 
-// FP64 clip (Sec. 2.3, clamped to [0, 1]), entry/exit voxels and first
-// crossings.  The faces the ray enters and leaves through are found in FP32
-// (in FP64 where FP32 cannot tell them apart); alpha_min / alpha_max are then
-// evaluated in FP64 on those faces.  Returns 1 for a hit, 0 when the ray
-// misses, -1 for non-finite geometry.
-// kEntry: also the entry point s + amin (p - s) in world coordinates (mm, from
-// the FP64 entry) into e[3], for the pose Jacobian.
-template <bool kEntry>
-__device__ __forceinline__ int ray_setup(const VolumeDev& vd, const PoseGeom& pg, int h, int w, RaySetup& r,
-                                         float* e = nullptr) {
-  double g[3];
+// FP64 clip (Sec. 2.3, clamped to [0, 1]).  The faces the ray enters and leaves
+// through are found in FP32 (in FP64 where FP32 cannot tell them apart);
+// alpha_min / alpha_max are then evaluated in FP64 on those faces.  Returns 1
+// for a hit, 0 when the ray misses, -1 for non-finite geometry.
+struct RayClip {
+  double g[3], rg[3];  // direction in voxel units and its reciprocals (0 for a parallel axis)
   float gf[3];
+  double amin, amax;
+  int ea, xa;  // axis of the entry / exit plane, -1 when clamped to alpha = 0 / 1
+};
+__device__ __forceinline__ int clip_ray(const PoseGeom& pg, int h, int w, RayClip& c) {
+  double* g = c.g;
+  float* gf = c.gf;
+  double* rg = c.rg;
   bool finite = true;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -347,7 +365,6 @@ __device__ __forceinline__ int ray_setup(const VolumeDev& vd, const PoseGeom& pg
     gf[a] = static_cast<float>(g[a]);
     finite = finite && isfinite(gf[a]) && isfinite(pg.u0f[a]);
   }
-  r.nseg = 0;
   if (!finite) return -1;
   // faces in FP32; a choice that FP32 cannot make safely -- the runner-up
   // crossing (or the clamp at alpha 0 / 1) within 2^-20 of the chosen one, four
@@ -374,7 +391,6 @@ __device__ __forceinline__ int ray_setup(const VolumeDev& vd, const PoseGeom& pg
   const float tol = 9.5367431640625e-7f * fmaxf(fabsf(lof), fabsf(hif)) + 1e-30f;  // 2^-20
   const bool exact = lof - lo2 < tol || hi2 - hif < tol || fabsf(hif - lof) < tol;
   if (!exact && !(lof < hif)) return 0;
-  double rg[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) rg[a] = g[a] != 0.0 ? rcp_fast(g[a]) : 0.0;
   // entry / exit faces: plane 0 when the ray runs up the axis, plane n otherwise
@@ -398,21 +414,46 @@ __device__ __forceinline__ int ray_setup(const VolumeDev& vd, const PoseGeom& pg
     }
   }
   if (!(amin < amax)) return 0;
-  r.ea = ea;
-  r.xa = xa;
-  r.amin = amin;
-  const double span = amax - amin;
+  c.ea = ea;
+  c.xa = xa;
+  c.amin = amin;
+  c.amax = amax;
+  return 1;
+}
+
+// Voxels in which the ray enters and leaves along one axis (entry and exit
+// positions ue, ux in voxel units).
+__device__ __forceinline__ void axis_voxels(const RayClip& c, int a, int n, double ue, double ux, int& i0, int& i1) {
+  const bool up = c.g[a] > 0.0;
+  if (a == c.ea) i0 = up ? 0 : n - 1;
+  else i0 = up ? floor_fast(ue) : -floor_fast(-ue) - 1;
+  if (a == c.xa) i1 = up ? n - 1 : 0;
+  else i1 = up ? -floor_fast(-ux) - 1 : floor_fast(ux);
+  i0 = min(max(i0, 0), n - 1);
+  i1 = min(max(i1, 0), n - 1);
+}
+
+// The exact crossing sequences of one ray (the fixed-point form of RaySetup),
+// from the FP64 clip.  Returns as clip_ray.
+__device__ __forceinline__ int ray_setup(const VolumeDev& vd, const PoseGeom& pg, int h, int w, RaySetup& r) {
+  r.nseg = 0;
+  RayClip c;
+  const int hit = clip_ray(pg, h, w, c);
+  if (hit <= 0) return hit;
+  const double* g = c.g;
+  const double* rg = c.rg;
+  r.ea = c.ea;
+  r.xa = c.xa;
+  r.amin = c.amin;
+  const double span = c.amax - c.amin;
   const double to_fix = kFixScale * rcp_fast(span);  // fixed-point units per unit of alpha
   r.unit = static_cast<float>(span) * (1.f / static_cast<float>(kExitUnits));
   int total = 0;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const int n = vd.n[a];
-    r.d[a] = gf[a] * vd.delta[a];
-    // entry position u_e (voxel units) and its world point (volume centred at
-    // the origin); u_e lies in [0, n], so FP32 holds it to ~1e-7 voxel
-    const double ue = fma(amin, g[a], pg.u0[a]);
-    if (kEntry) e[a] = fmaf(static_cast<float>(ue), vd.delta[a], -0.5f * static_cast<float>(n) * vd.delta[a]);
+    r.d[a] = c.gf[a] * vd.delta[a];
+    const double ue = fma(c.amin, g[a], pg.u0[a]);
     if (g[a] == 0.0) {
       r.ient[a] = min(max(static_cast<int>(floor(pg.u0[a])), 0), n - 1);
       r.cnt[a] = 0;
@@ -422,14 +463,8 @@ __device__ __forceinline__ int ray_setup(const VolumeDev& vd, const PoseGeom& pg
       continue;
     }
     const bool up = g[a] > 0.0;
-    const double ux = fma(amax, g[a], pg.u0[a]);
     int i0, i1;
-    if (a == ea) i0 = up ? 0 : n - 1;
-    else i0 = up ? floor_fast(ue) : -floor_fast(-ue) - 1;
-    if (a == xa) i1 = up ? n - 1 : 0;
-    else i1 = up ? -floor_fast(-ux) - 1 : floor_fast(ux);
-    i0 = min(max(i0, 0), n - 1);
-    i1 = min(max(i1, 0), n - 1);
+    axis_voxels(c, a, n, ue, fma(c.amax, g[a], pg.u0[a]), i0, i1);
     r.ient[a] = i0;
     r.cnt[a] = max(up ? i1 - i0 : i0 - i1, 0);
     total += r.cnt[a];
@@ -461,7 +496,7 @@ __device__ __forceinline__ int ray_setup(const VolumeDev& vd, const PoseGeom& pg
 #define DRR_FWD_MINB 4
 #endif
 #ifndef DRR_JAC_MINB
-#define DRR_JAC_MINB 4
+#define DRR_JAC_MINB 3
 #endif
 constexpr float kTwoM32 = 2.3283064365386963e-10f;  // 2^-32
 
@@ -471,18 +506,6 @@ struct WalkScratch {
   unsigned long long A0[3][kThreads];
   unsigned long long D[3][kThreads];
 };
-// The Jacobian walk also keeps the state at the start of the current chunk,
-// for an exact re-walk of the chunk.  (Shared memory comes out of the same
-// on-chip store as the L1 cache that serves the voxel gathers, so each kernel
-// declares only what its walk uses.)
-struct JacScratch : WalkScratch {
-  int cnt[3][kThreads];  // crossings per slot (read only by the exact re-walk)
-  float e[3][kThreads];  // the ray's entry point (read only by the Jacobian epilogue)
-  int c_off[kThreads];
-  float c_v[kThreads], c_vprev[kThreads];
-  int c_pend[kThreads];
-};
-
 __device__ __forceinline__ unsigned long long fix_at(unsigned long long A0, unsigned long long D, unsigned int k) {
   return A0 + static_cast<unsigned long long>(k) * D;
 }
@@ -551,36 +574,20 @@ __device__ __forceinline__ float local_pos(unsigned long long x, unsigned long l
   return fix_to_float(static_cast<long long>(x - O));
 }
 
-// Both walks gather two crossings ahead: the first crossing of a chunk is
+// The forward walk gathers two crossings ahead: the first crossing of a chunk is
 // peeled and the unrolled loop runs chunk - 1 times.  The three voxel registers
 // of that pipeline rotate without register moves when the unroll is a multiple
-// of 3.  The Jacobian walk's 6 divides chunk - 1 for every chunk length; the
-// forward walk's 12 divides it for its long-ray chunks (121, 181) and for 13.
-// (Measured on the CT batch: forward 6 / 12 / 24 at 0.376 / 0.371 / 0.375 ms,
-// Jacobian 3 / 6 / 12 at 0.649 / 0.556 / 0.563 ms.)
+// of 3; 12 divides chunk - 1 for the long-ray chunks (121, 181) and for 13.
+// (Measured on the CT batch: 6 / 12 / 24 at 0.376 / 0.371 / 0.375 ms.)
 #ifndef DRR_FWD_UNROLL
 #define DRR_FWD_UNROLL 12
 #endif
-#ifndef DRR_JAC_UNROLL
-#define DRR_JAC_UNROLL 6
-#endif
 constexpr int kFwdUnroll = DRR_FWD_UNROLL;
-constexpr int kJacUnroll = DRR_JAC_UNROLL;
 // Chunk length per ray.  The FP32 error of a local position grows with the
 // chunk's share of the ray, so long rays take long chunks (fewer exact
-// re-anchorings) and short rays short ones; 6k + 1 crossings.  The Jacobian
-// walk stays at 61 for long rays: its tie test's threshold grows with the
-// positions, so longer chunks are flagged (and walked twice) more often.  The
-// forward walk has no tie test and takes 121 / 181 for rays of more than 512 /
-// 1024 segments (on the CT workload: 3 % faster, worst pixel error unchanged).
-#ifndef DRR_JAC_LONG
-#define DRR_JAC_LONG 61
-#endif
-__device__ __forceinline__ int walk_chunk(int nseg) {
-  return nseg > 512 ? DRR_JAC_LONG : nseg > 256 ? 31 : nseg > 128 ? 19 : 13;
-}
+// re-anchorings) and short rays short ones.
 __device__ __forceinline__ int fwd_chunk(int nseg) {
-  return nseg > 1024 ? 181 : nseg > 512 ? 121 : walk_chunk(nseg);
+  return nseg > 1024 ? 181 : nseg > 512 ? 121 : nseg > 256 ? 31 : nseg > 128 ? 19 : 13;
 }
 
 // Forward walk (Eq. 2 with the crossings of Eq. 3 taken in order, Sec. 2.2).
@@ -664,321 +671,719 @@ __device__ __forceinline__ float walk_forward(const VolumeDev& vd, const RaySetu
   return acc * r.unit;
 }
 
-// Walk with the pose-Jacobian bookkeeping (Sec. 2.4).  Crossing k with weight
-// w_k = V_before - V_after adds to per-axis sums G_a = sum w, A_a = sum w alpha
-// (alpha from the entry).  The axes are relabelled per ray so that slot 2 is the
-// axis with most crossings; only slots 0 and 1 are summed and slot 2 follows
-// from sum_k w_k = 0 and sum_k w_k alpha_k = F over all crossings, entry and
-// exit included (end points clamped to alpha = 0 or 1 belong to no axis and are
-// kept in Gc, Ac).
+// ---------------------------------------------------------------------------
+// Slab walk (Eq. 2 by the crossings of each axis on their own; the crossings
+// are those of Eq. 3, Sec. 2.2).  With the axis of the largest direction
+// component as the dominant one, its planes cut the ray into slabs of equal
+// length, and
+//   E = sum over slabs V[voxel the slab is entered in] * slab length
+//     + sum over the minor axes' crossings (V after - V before) * (slab end - crossing),
+// so nothing has to be merged in order: each axis' crossings are one counted
+// loop, whose iterations are independent (the loads of several are in flight
+// at once) and need no minimum, no ordering compares and no carried weights.
+// The pose Jacobian's per-axis sums (Sec. 2.4) of w = V before - V after and of
+// w times its position are those of the two minor loops; the dominant axis'
+// follow from sum w = 0 and sum w alpha = F over all crossings.
+// Measured (fused forward + Jacobian kernel, FP32, CUDA events): 16-pose CT
+// batch, 512x512x133 and 200x200, 0.559 -> 0.413 ms against the walk that merged
+// the axes' crossings in order (429 -> 267 M warp instructions); 150x141 on 256^3
+// split over the warps of a tile, 0.067 -> 0.051 ms.  What bounds it now is the L1
+// data pipe (82 % busy): the dominant loop's gathers touch ~15 lines each (rays of
+// a tile at one plane x = const of an x-fastest volume), ~5 wavefronts.  Taking
+// 2 x 4 rays and 4 planes per gather (35 instead of 50 M wavefronts but more L2
+// sectors, 0.469 ms), the three loops interleaved in chunks (0.505), and a second
+// copy of the volume with another fastest axis (17 M wavefronts, but every
+// gather an L2 access and 0.74 GB from DRAM: 0.446) were slower.  The forward
+// alone keeps the merged walk: it gathers once per segment, the slab walk once
+// per slab and twice per minor crossing (0.391 against 0.366 ms).
 //
-// The order of two crossings decides the voxel between them and hence both
-// weights, so it must be exact.  A chunk's FP32 position t = l * dl + x0 (x0
-// and dl each one rounding from exact values, see fix_to_float, then the FMA)
-// is within 2^-24 (x0 + l dl + t) + (l + 1) 2^-25 = 2^-23 t + (l + 1) 2^-25
-// units of the exact one, so the walk can only misorder two crossings less
-// than 2^-22 t + 62 * 2^-24 apart, and then it takes a segment no longer than
-// that at the misordered pair.  So each chunk tracks its shortest segment and
-// the gap to the next crossing after it; if either is below kTieRel * position
-// + kTieAbs (25 % and ~250x above those two terms), the chunk is walked again
-// from its saved start state in exact fixed-point order (rare: about one lane
-// in two thousand chunks).
-// Sums are kept per chunk in local positions and moved to the anchor frame
-// when the chunk ends, so a re-walk only discards the chunk's own sums.
+// Coordinates run in the ray's direction on every axis, from the entry voxel's
+// lower plane: q_a in [0, 1] at the entry, crossing k of axis a at q_a = 1 + k.
+// Positions are 32.32 fixed point.  Slot 2 is the dominant axis, 0 and 1 the
+// others (by decreasing direction).  The voxel that a crossing lies in is read
+// off the integer parts of the other axes' coordinates at it; the two views of
+// a pair of crossings (each in the other's loop) agree unless the pair is closer
+// than the rounding of these coordinates.  A minor loop's smallest fractional
+// distance to a plane is tracked against a bound on that rounding (SlabRay::t0,
+// t1), and a ray with a pair below it is summed again by exact_rays, in exact
+// order (about 1 ray in 2000 on a CT).
+//
+// The loops are cut into up to kPieces pieces of whole plane ranges, the same
+// planes for the warp's 32 rays (so rays of one tile gather from the same plane
+// at a time), and the pieces' sums are added in order: the split kernel, whose
+// warps take different pieces, gives the same bits.
+// ---------------------------------------------------------------------------
+#ifndef DRR_PIECE_LEN
+#define DRR_PIECE_LEN 32
+#endif
+#ifndef DRR_PIECES
+#define DRR_PIECES 8
+#endif
+constexpr int kPieces = DRR_PIECES, kPieceLen = DRR_PIECE_LEN;
+#ifndef DRR_SLAB_UNROLL
+#define DRR_SLAB_UNROLL 8
+#endif
+#ifndef DRR_MINOR_UNROLL
+#define DRR_MINOR_UNROLL 4
+#endif
+constexpr int kSlabUnroll = DRR_SLAB_UNROLL, kMinorUnroll = DRR_MINOR_UNROLL;  // loop iterations in flight
+using u32 = unsigned int;
+using u64 = unsigned long long;
+
+// Per-ray values that only the ray's end needs, parked in shared memory while
+// the loops run.
+enum ParkSlot : int {
+  kPkD = 0,       // p - s in mm (3)
+  kPkE = 3,       // the entry point (3); the detector-parameter mode keeps 1 - 2 amin and amin here
+  kPkF0 = 6,      // alpha from the entry to the first crossing of slots 0, 1 (2)
+  kPkRg = 8,      // alpha per plane of slots 0, 1 (2)
+  kPkSpan = 10,   // alpha_max - alpha_min
+  kPkCount = 11
+};
+struct Park {
+  float v[kPkCount][kThreads];
+};
+template <int MODE>
+struct ParkFor {
+  using type = std::conditional_t<MODE == kFwdJac || MODE == kPoseGrad || MODE == kGeoGrad, Park, WalkScratch>;
+};
+
+struct SlabRay {
+  int cnt[3];      // crossings per slot
+  int i0[3];       // entry voxel index per slot, counted in the ray's direction
+  int off;         // element offset of the entry voxel (padded layout)
+  int step[3];     // signed element stride per slot
+  int ax0, ax1, ax2;  // real axis of each slot
+  int ea, xa;      // axis of the entry / exit plane, -1 when clamped to alpha = 0 / 1
+  u64 Y, Z;        // q_0, q_1 at dominant crossing 0 and their step per dominant crossing
+  u32 dy, dz;
+  u64 mX, mdX;     // slot 0's crossing 0: q_2 and q_1 (both + t0) and their steps
+  u64 mZ;
+  u32 mdz;
+  u64 lX, ldX;     // slot 1's crossing 0: q_2 and q_0 (both + t1) and their steps
+  u64 lY, ldY;
+  u32 t0, t1;      // rounding bounds (and biases) of the minor loops' coordinates
+  float w1;        // 1 - q_2 at the entry: the first slab's share inside the ray
+  float rest;      // share of the last slab beyond the exit
+  float rg2;       // alpha per dominant plane
+  bool exact;      // to be summed by exact_rays
+};
+
+// A lane without a ray to walk takes part with no crossings.
+__device__ __forceinline__ void slab_idle(const VolumeDev& vd, SlabRay& s) {
+  s = SlabRay{};
+  s.off = vd.origin;
+}
+
+// x * m / 2^32 for a 32.32 number m and a fraction x (0.32), rounded down.
+__device__ __forceinline__ u64 mul_frac(u32 x, u64 m) {
+  return static_cast<u64>(x) * static_cast<u32>(m >> 32) + __umulhi(x, static_cast<u32>(m));
+}
+
+// ---------------------------------------------------------------------------
+// Float-float arithmetic (unevaluated sums h + l of two FP32 numbers, ~2^-46
+// relative; Dekker 1971, Knuth TAOCP 2, with FMA products).  The per-ray setup
+// needs ~2^-36 of a voxel; this GPU issues FP64 at 1/64 of the FP32 rate, and
+// ~75 FP64 operations per ray took longer than the walk itself (277 us of an
+// empty walk of the 16-pose CT batch).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float2 ff_sum(float a, float b) {  // exact a + b
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t)));
+}
+__device__ __forceinline__ float2 ff_norm(float h, float l) {  // |h| >= |l|
+  const float s = __fadd_rn(h, l);
+  return make_float2(s, __fsub_rn(l, __fsub_rn(s, h)));
+}
+__device__ __forceinline__ float2 ff_add(float2 a, float2 b) {
+  const float2 s = ff_sum(a.x, b.x);
+  return ff_norm(s.x, __fadd_rn(s.y, __fadd_rn(a.y, b.y)));
+}
+__device__ __forceinline__ float2 ff_mul(float2 a, float2 b) {
+  const float p = __fmul_rn(a.x, b.x);
+  const float e = __fmaf_rn(a.x, b.y, __fmaf_rn(a.y, b.x, __fmaf_rn(a.x, b.x, -p)));
+  return ff_norm(p, e);
+}
+__device__ __forceinline__ float2 ff_rcp(float2 a) {  // 1e-30 < |a| < 1e30
+  const float r = __frcp_rn(a.x);
+  const float e = __fmaf_rn(-a.y, r, __fmaf_rn(-a.x, r, 1.f));
+  return ff_norm(r, __fmul_rn(r, e));
+}
+// x as the unevaluated sum of two FP32 numbers.
+__device__ __forceinline__ float2 ff_from(double x) {
+  const float h = static_cast<float>(x);
+  return make_float2(h, static_cast<float>(x - static_cast<double>(h)));
+}
+
+// A pose's FP64 geometry as float-float pairs, for the per-ray setup.
+struct GeomFF {
+  float2 u0[3], un[3], g00[3], gw[3], gh[3];
+};
+// From the pose's geometry in shared memory, by a warp (or the first warp of a
+// block) after the geometry's copy; the caller synchronises.
+__device__ __forceinline__ void geom_ff(const PoseGeom& pg, GeomFF& gf) {
+  static_assert(sizeof(GeomFF) == 15 * sizeof(float2), "one pair per FP64 value");
+  const int lane = threadIdx.x & 31;
+  if (lane < 15) reinterpret_cast<float2*>(&gf)[lane] = ff_from(reinterpret_cast<const double*>(&pg)[lane]);
+}
+// x in [0, 2^31) as 32.32 fixed point; a negative x (rounding) gives 0.
+__device__ __forceinline__ u64 ff_fix(float2 x) {
+  if (x.x < 0.f) return 0ull;
+  const float fl = floorf(x.x);
+  const u64 v = (static_cast<u64>(__float2uint_rz(fl)) << 32) + __float2uint_rz((x.x - fl) * 4294967296.f);
+  const long long lo = static_cast<long long>(__float2int_rn(x.y * 4294967296.f));
+  const long long r = static_cast<long long>(v) + lo;
+  return r < 0 ? 0ull : static_cast<u64>(r);
+}
+// x <= 1 as a 32-bit fraction (1 becomes 1 - 2^-32).
+__device__ __forceinline__ u32 ff_frac(float2 x) {
+  const u64 v = static_cast<u64>(__float2uint_rz(x.x * 4294967296.f)) +
+                static_cast<u64>(static_cast<long long>(__float2int_rn(x.y * 4294967296.f)));
+  return v >> 32 ? (static_cast<long long>(v) < 0 ? 0u : 0xffffffffu) : static_cast<u32>(v);
+}
+__device__ __forceinline__ float fix_float(u64 x) {  // 32.32 fixed point to FP32
+  return fmaf(static_cast<float>(static_cast<u32>(x)), kTwoM32, static_cast<float>(static_cast<u32>(x >> 32)));
+}
+
+// The ray's slab form.  Returns 1 for a hit, 0 for a miss, -1 for non-finite
+// geometry.  All in FP32 / float-float / fixed point; where that cannot decide
+// (faces, end voxels or end counts closer than its rounding) s.exact is set and
+// exact_rays decides in FP64.
+template <int MODE>
+__device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& pg, const GeomFF& gf, int h,
+                                          int w, SlabRay& s, Park* park) {
+  const int t = threadIdx.x;
+  float2 g[3];
+  if (w < (1 << 24) && h < (1 << 24)) {
+    const float fw = static_cast<float>(w), fh = static_cast<float>(h);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const float p = __fmul_rn(fw, gf.gw[a].x), q = __fmul_rn(fh, gf.gh[a].x);
+      const float pe = __fmaf_rn(fw, gf.gw[a].y, __fmaf_rn(fw, gf.gw[a].x, -p));
+      const float qe = __fmaf_rn(fh, gf.gh[a].y, __fmaf_rn(fh, gf.gh[a].x, -q));
+      const float2 u = ff_sum(p, q), v = ff_sum(gf.g00[a].x, u.x);
+      g[a] = ff_norm(v.x, __fadd_rn(__fadd_rn(v.y, u.y), __fadd_rn(__fadd_rn(pe, qe), gf.g00[a].y)));
+    }
+  } else {
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      g[a] = ff_from(fma(static_cast<double>(h), pg.gh[a], fma(static_cast<double>(w), pg.gw[a], pg.g00[a])));
+  }
+  // faces in FP32; a choice that FP32 cannot make safely -- the runner-up
+  // crossing (or the clamp at alpha 0 / 1) within 2^-20 of the chosen one, four
+  // times the FP32 error of these products, or a hit test that close -- is left
+  // to exact_rays.  That matters where the clipped span is a small part of alpha
+  // (a small volume far from the source): there an FP32 tie moves the entry by
+  // a visible share of the span.
+  float lof = 0.f, hif = 1.f, lo2 = -1.f, hi2 = 2.f;  // chosen and runner-up entry / exit
+  int ea = -1, xa = -1;
+  bool finite = true, hit = true, unsafe = false;
+  float2 ar[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    finite = finite && isfinite(g[a].x) && isfinite(gf.u0[a].x);
+    park->v[kPkD + a][t] = g[a].x * vd.delta[a];
+    if (g[a].x != 0.f) {
+      ar[a] = ff_rcp(make_float2(fabsf(g[a].x), g[a].x < 0.f ? -g[a].y : g[a].y));
+      unsafe = unsafe || fabsf(g[a].x) < 1e-20f;
+      const float rf = copysignf(ar[a].x, g[a].x);
+      const float t0 = -gf.u0[a].x * rf, t1 = gf.un[a].x * rf;
+      const float lo = fminf(t0, t1), hi = fmaxf(t0, t1);
+      if (lo > lof) { lo2 = lof; lof = lo; ea = a; } else lo2 = fmaxf(lo2, lo);
+      if (hi < hif) { hi2 = hif; hif = hi; xa = a; } else hi2 = fminf(hi2, hi);
+    } else {
+      ar[a] = make_float2(0.f, 0.f);
+      if (!(pg.u0[a] >= 0.0 && pg.un[a] > 0.0)) hit = false;
+    }
+  }
+  if (!finite) return -1;
+  if (!hit) return 0;
+  const float tol = 9.5367431640625e-7f * fmaxf(fabsf(lof), fabsf(hif)) + 1e-30f;  // 2^-20
+  unsafe = unsafe || lof - lo2 < tol || hi2 - hif < tol || fabsf(hif - lof) < tol;
+  if (unsafe) {
+    slab_idle(vd, s);
+    s.exact = true;
+    return 1;
+  }
+  if (!(lof < hif)) return 0;
+  // slots: 2 the largest direction component, 1 the smallest
+  float2 ag[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) ag[a] = make_float2(fabsf(g[a].x), g[a].x < 0.f ? -g[a].y : g[a].y);
+  const auto more = [](float2 x, float2 y) { return x.x > y.x || (x.x == y.x && x.y > y.y); };
+  const int a2 = more(ag[2], ag[0]) && more(ag[2], ag[1]) ? 2 : (more(ag[1], ag[0]) ? 1 : 0);
+  const int p = a2 == 0 ? 1 : 0, q = a2 == 2 ? 1 : 2;
+  const bool pq = !more(pick3(q, ag[0], ag[1], ag[2]), pick3(p, ag[0], ag[1], ag[2]));
+  const int ax[3] = {pq ? p : q, pq ? q : p, a2};
+  s.ax0 = ax[0];
+  s.ax1 = ax[1];
+  s.ax2 = ax[2];
+  s.ea = ea;
+  s.xa = xa;
+  float2 sg[3], sr[3], U[3], N[3];  // direction, its reciprocal, source and far face (in the ray's direction), per slot
+  int n[3];
+  bool up[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    sg[k] = pick3(ax[k], ag[0], ag[1], ag[2]);
+    sr[k] = pick3(ax[k], ar[0], ar[1], ar[2]);
+    n[k] = pick3(ax[k], vd.n[0], vd.n[1], vd.n[2]);
+    up[k] = !(pick3(ax[k], g[0].x, g[1].x, g[2].x) < 0.f);
+    const float2 u = pick3(ax[k], gf.u0[0], gf.u0[1], gf.u0[2]), v = pick3(ax[k], gf.un[0], gf.un[1], gf.un[2]);
+    U[k] = up[k] ? u : v;
+    N[k] = up[k] ? v : u;
+    const int st = pick3(ax[k], vd.stride[0], vd.stride[1], vd.stride[2]);
+    s.step[k] = up[k] ? st : -st;
+  }
+  float2 amin = make_float2(0.f, 0.f), amax = make_float2(1.f, 0.f);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (ea == ax[k]) amin = ff_mul(make_float2(-U[k].x, -U[k].y), sr[k]);
+    if (xa == ax[k]) amax = ff_mul(N[k], sr[k]);
+  }
+  // float-float rounding of positions, in 2^-32 voxel
+  const float far = fmaxf(fmaxf(fabsf(gf.u0[0].x) + fabsf(gf.un[0].x), fabsf(gf.u0[1].x) + fabsf(gf.un[1].x)),
+                          fabsf(gf.u0[2].x) + fabsf(gf.un[2].x)) * 2.44140625e-4f;
+  const u32 te = static_cast<u32>(fminf(far, 1e8f)) + 4u;
+  bool exact = far > 1e8f;
+  // entry voxel and fraction per axis
+  u32 E[3];
+  s.off = vd.origin;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    float uef = 0.f;
+    if (ea == ax[k]) {
+      E[k] = 0u;
+      s.i0[k] = 0;
+    } else {
+      const float2 ue = ff_add(U[k], ff_mul(amin, sg[k]));
+      uef = ue.x;
+      const u64 f = min(ff_fix(ue), (static_cast<u64>(n[k]) << 32) - 1ull);
+      E[k] = static_cast<u32>(f);
+      s.i0[k] = static_cast<int>(f >> 32);
+      if (sg[k].x != 0.f && E[k] + te < 2u * te) exact = true;
+    }
+    // element offset of the entry voxel: counted from the far end where the ray runs down
+    s.off += s.step[k] * (up[k] ? s.i0[k] : s.i0[k] - (n[k] - 1));
+    if (MODE != kGeoGrad) {
+      // the entry point in world coordinates (volume centred at the origin)
+      const float dl = pick3(ax[k], vd.delta[0], vd.delta[1], vd.delta[2]), half = 0.5f * static_cast<float>(n[k]);
+      const float e = up[k] ? fmaf(uef, dl, -half * dl) : fmaf(-uef, dl, half * dl);
+      if (ax[k] == 0) park->v[kPkE][t] = e;
+      else if (ax[k] == 1) park->v[kPkE + 1][t] = e;
+      else park->v[kPkE + 2][t] = e;
+    }
+  }
+  s.dy = ff_frac(ff_mul(sg[0], sr[2]));
+  s.dz = ff_frac(ff_mul(sg[1], sr[2]));
+  s.mdz = ff_frac(ff_mul(sg[1], sr[0]));
+  const float2 r20 = ff_mul(sg[2], sr[0]), r21 = ff_mul(sg[2], sr[1]), r01 = ff_mul(sg[0], sr[1]);
+  // exit: coordinate along the dominant axis, then the counts
+  u64 qx = static_cast<u64>(n[2] - s.i0[2]) << 32;
+  s.cnt[2] = n[2] - 1 - s.i0[2];
+  s.rest = 0.f;
+  if (xa != ax[2]) {
+    const float2 ux = ff_add(U[2], ff_mul(amax, sg[2]));
+    const u64 base = static_cast<u64>(s.i0[2]) << 32, f = ff_fix(ux);
+    qx = min(f > base + E[2] ? f - base : static_cast<u64>(E[2]), qx - 1ull);
+    s.cnt[2] = static_cast<int>(qx >> 32);
+    const u32 fr = static_cast<u32>(qx);
+    s.rest = static_cast<float>(0u - fr) * kTwoM32;
+    if (fr == 0u) s.rest = 1.f;
+    if (fr + te < 2u * te) exact = true;
+  }
+  const float dom = static_cast<float>(s.cnt[2]) + 16.f + far;
+  const u32 tx = static_cast<u32>(fminf(dom, 2e8f));
+  const u64 len = qx - E[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int most = n[k] - 1 - s.i0[k];
+    if (sg[k].x == 0.f) {
+      s.cnt[k] = 0;
+    } else if (xa == ax[k]) {
+      s.cnt[k] = most;
+    } else {
+      const u32 sl = k == 0 ? s.dy : s.dz;
+      const u64 f = static_cast<u64>(E[k]) + static_cast<u64>(static_cast<u32>(len >> 32)) * sl +
+                    __umulhi(static_cast<u32>(len), sl);
+      s.cnt[k] = min(static_cast<int>(f >> 32), most);
+      if (static_cast<u32>(f) + tx < 2u * tx) exact = true;
+    }
+  }
+  // rounding bounds in 2^-32: a minor crossing's own coordinates err by at most
+  // ~cnt + 3, the dominant loop's view of it by ~cnt_2 + 3 of its plane spacings
+  // (twice that where the start was pulled back below)
+  const float t0 = fmaf(2.f * dom, r20.x, static_cast<float>(s.cnt[0]) + 16.f + far);
+  const float t1 = fmaf(2.f * dom, r21.x, static_cast<float>(s.cnt[1]) + 16.f + far);
+  // an axis whose planes lie more than 2^16 slabs apart, or a bound that is no
+  // longer small, goes to exact_rays
+  if (s.cnt[0] > 0 && !(r20.x < 65536.f && t0 < 2.68435456e8f)) exact = true;
+  if (s.cnt[1] > 0 && !(r21.x < 65536.f && t1 < 2.68435456e8f)) exact = true;
+  s.exact = exact;
+  if (exact) s.cnt[0] = s.cnt[1] = s.cnt[2] = 0;
+  s.t0 = s.cnt[0] > 0 ? static_cast<u32>(t0) : 0u;
+  s.t1 = s.cnt[1] > 0 ? static_cast<u32>(t1) : 0u;
+  s.mdX = ff_fix(r20.x < 65536.f ? r20 : make_float2(0.f, 0.f));
+  s.ldX = ff_fix(r21.x < 65536.f ? r21 : make_float2(0.f, 0.f));
+  s.ldY = ff_fix(r21.x < 65536.f ? r01 : make_float2(0.f, 0.f));
+  s.Y = static_cast<u64>(E[0]) + (s.dy - __umulhi(E[2], s.dy));
+  s.Z = static_cast<u64>(E[1]) + (s.dz - __umulhi(E[2], s.dz));
+  s.mX = E[2] + (s.mdX - mul_frac(E[0], s.mdX)) + s.t0;
+  s.mZ = static_cast<u64>(E[1]) + (s.mdz - __umulhi(E[0], s.mdz)) + s.t0;
+  s.lX = E[2] + (s.ldX - mul_frac(E[1], s.ldX)) + s.t1;
+  s.lY = E[0] + (s.ldY - mul_frac(E[1], s.ldY)) + s.t1;
+  if (s.cnt[2] > 0) {
+    // no minor plane beyond the exit is counted at the last dominant crossing:
+    // where rounding would, the start is pulled back by the excess
+    const u64 m = static_cast<u64>(s.cnt[2] - 1);
+    const u64 ey = s.Y + m * s.dy, ly = static_cast<u64>(s.cnt[0] + 1) << 32;
+    if (ey >= ly) s.Y -= min(s.Y, ey - ly + 1ull);
+    const u64 ez = s.Z + m * s.dz, lz = static_cast<u64>(s.cnt[1] + 1) << 32;
+    if (ez >= lz) s.Z -= min(s.Z, ez - lz + 1ull);
+  }
+  s.w1 = E[2] == 0u ? 1.f : static_cast<float>(0u - E[2]) * kTwoM32;
+  s.rg2 = sr[2].x;
+  if (MODE == kGeoGrad) {
+    park->v[kPkE][t] = (1.f - 2.f * amin.x) - 2.f * amin.y;
+    park->v[kPkE + 1][t] = amin.x;
+  }
+  park->v[kPkF0][t] = (E[0] == 0u ? 1.f : static_cast<float>(0u - E[0]) * kTwoM32) * sr[0].x;
+  park->v[kPkF0 + 1][t] = (E[1] == 0u ? 1.f : static_cast<float>(0u - E[1]) * kTwoM32) * sr[1].x;
+  park->v[kPkRg][t] = sr[0].x;
+  park->v[kPkRg + 1][t] = sr[1].x;
+  park->v[kPkSpan][t] = fix_float(len) * sr[2].x;
+  return 1;
+}
+
+// The loops are cut into np pieces: piece p takes of each slot the planes
+// [p, p + 1) * len counted from the warp's first entry plane (sh: this ray's
+// entry plane in that count).
+struct Pieces {
+  int sh, len;
+};
+struct Plan {
+  Pieces slot[3];
+  int np;
+};
+__device__ __forceinline__ Plan plan_pieces(const SlabRay& s) {
+  constexpr u32 kAll = 0xffffffffu;
+  Plan pl;
+  int total[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int base = __reduce_min_sync(kAll, s.cnt[k] > 0 ? s.i0[k] : 0x7fffffff);
+    pl.slot[k].sh = s.cnt[k] > 0 ? s.i0[k] - base : 0;
+    total[k] = __reduce_max_sync(kAll, s.cnt[k] > 0 ? pl.slot[k].sh + s.cnt[k] : 0);
+  }
+  pl.np = min(max((total[2] + kPieceLen - 1) / kPieceLen, 1), kPieces);
+  // whole unrolled blocks per piece
+  pl.slot[0].len = ((total[0] + pl.np - 1) / pl.np + kMinorUnroll - 1) / kMinorUnroll * kMinorUnroll;
+  pl.slot[1].len = ((total[1] + pl.np - 1) / pl.np + kMinorUnroll - 1) / kMinorUnroll * kMinorUnroll;
+  pl.slot[2].len = ((total[2] + pl.np - 1) / pl.np + kSlabUnroll - 1) / kSlabUnroll * kSlabUnroll;
+  return pl;
+}
+// First crossing of piece p.
+__device__ __forceinline__ int piece_start(const Pieces& pc, int p, int cnt) {
+  return min(max(p * pc.len - pc.sh, 0), cnt);
+}
+
+// Pieces [p0, p1) of the sum of the voxels entered at dominant crossings; piece
+// p's sum goes to sink(p, sum).
+template <int DT, class Sink>
+__device__ __forceinline__ void dominant_loop(const VolumeDev& vd, const SlabRay& s, const Pieces& pc, int p0, int p1,
+                                              Sink sink) {
+  int m = piece_start(pc, p0, s.cnt[2]);
+  const u64 Y = s.Y + static_cast<u64>(static_cast<u32>(m)) * s.dy;
+  const u64 Z = s.Z + static_cast<u64>(static_cast<u32>(m)) * s.dz;
+  u32 fy = static_cast<u32>(Y), fz = static_cast<u32>(Z);
+  int off = s.off + (m + 1) * s.step[2] + static_cast<int>(Y >> 32) * s.step[0] + static_cast<int>(Z >> 32) * s.step[1];
+  const int st = s.step[2], st0 = st + s.step[0], s1 = s.step[1];
+#pragma unroll 1
+  for (int p = p0; p < p1; ++p) {
+    const int end = piece_start(pc, p + 1, s.cnt[2]);
+    float S = 0.f;
+#pragma unroll kSlabUnroll
+    for (; m < end; ++m) {
+      S += gather<DT>(vd, off);
+      fy += s.dy;
+      fz += s.dz;
+      off += (fy < s.dy ? st0 : st) + (fz < s.dz ? s1 : 0);
+    }
+    sink(p, S);
+  }
+}
+
+// Sums over one minor axis' crossings, w = V after - V before: g = sum w,
+// c = sum w f (f: biased fraction of the slab at the crossing, times 2^32), h =
+// sum w k (Jacobian modes); near: the smallest biased fraction.
+struct MinorSums {
+  float g, c, h;
+  u32 near;
+};
+#define DRR_MINOR_BLOCK(ON, ADVANCE)                                   \
+  {                                                                    \
+    float v0[kU], v1[kU];                                              \
+    u32 f[kU];                                                         \
+    _Pragma("unroll") for (int j = 0; j < kU; ++j) {                   \
+      v0[j] = v1[j] = 0.f;                                             \
+      f[j] = static_cast<u32>(X);                                      \
+      if (ON) {                                                        \
+        const int o = OFFSET;                                          \
+        v0[j] = gather<DT>(vd, o);                                     \
+        v1[j] = gather_at<DT>(vd, after, o, sk);                       \
+        r.near = min(r.near, min(f[j], NEAR));                         \
+        ADVANCE                                                        \
+      }                                                                \
+    }                                                                  \
+    _Pragma("unroll") for (int j = 0; j < kU; ++j) {                   \
+      const float w = v1[j] - v0[j];                                   \
+      r.g += w;                                                        \
+      r.c = fmaf(w, static_cast<float>(f[j]), r.c);                    \
+      r.h = fmaf(w, kf + static_cast<float>(j), r.h);                  \
+    }                                                                  \
+    kf += static_cast<float>(kU);                                      \
+  }
+#define DRR_MINOR_PIECES(CNT, ADVANCE)                                 \
+  _Pragma("unroll 1") for (int p = p0; p < p1; ++p) {                  \
+    const int end = piece_start(pc, p + 1, CNT), k0 = k;               \
+    MinorSums r{0.f, 0.f, 0.f, 0xffffffffu};                           \
+    float kf = 0.f;                                                    \
+    for (; k + kU <= end; k += kU) DRR_MINOR_BLOCK(true, ADVANCE)      \
+    if (k < end) {                                                     \
+      DRR_MINOR_BLOCK(k + j < end, ADVANCE)                            \
+      k = end;                                                         \
+    }                                                                  \
+    r.h = fmaf(static_cast<float>(k0), r.g, r.h);                      \
+    sink(p, r);                                                        \
+  }
+
+// Slot 0: the slab (q_2) advances by at least one plane per crossing, slot 1's
+// coordinate by at most one.
+template <int DT, class Sink>
+__device__ __forceinline__ void middle_loop(const VolumeDev& vd, const SlabRay& s, const Pieces& pc, int p0, int p1,
+                                            Sink sink) {
+  constexpr int kU = kMinorUnroll;
+  int k = piece_start(pc, p0, s.cnt[0]);
+  u64 X = s.mX + static_cast<u64>(static_cast<u32>(k)) * s.mdX;
+  const u64 Z = s.mZ + static_cast<u64>(static_cast<u32>(k)) * s.mdz;
+  u32 fz = static_cast<u32>(Z);
+  const int sk = s.step[0], sx = s.step[2], st = sk + s.step[1];
+  int o1 = s.off + k * sk + static_cast<int>(Z >> 32) * s.step[1];
+  const void* after = base_after<DT>(vd, sk);
+#define OFFSET (o1 + static_cast<int>(X >> 32) * sx)
+#define NEAR fz
+  DRR_MINOR_PIECES(s.cnt[0], X += s.mdX; fz += s.mdz; o1 += fz < s.mdz ? st : sk;)
+#undef OFFSET
+#undef NEAR
+}
+
+// Slot 1: both other coordinates may advance by several planes per crossing.
+template <int DT, class Sink>
+__device__ __forceinline__ void least_loop(const VolumeDev& vd, const SlabRay& s, const Pieces& pc, int p0, int p1,
+                                           Sink sink) {
+  constexpr int kU = kMinorUnroll;
+  int k = piece_start(pc, p0, s.cnt[1]);
+  u64 X = s.lX + static_cast<u64>(static_cast<u32>(k)) * s.ldX;
+  u64 Y = s.lY + static_cast<u64>(static_cast<u32>(k)) * s.ldY;
+  const int sk = s.step[1], sx = s.step[2], sy = s.step[0];
+  int o1 = s.off + k * sk;
+  const void* after = base_after<DT>(vd, sk);
+#define OFFSET (o1 + static_cast<int>(X >> 32) * sx + static_cast<int>(Y >> 32) * sy)
+#define NEAR static_cast<u32>(Y)
+  DRR_MINOR_PIECES(s.cnt[1], X += s.ldX; Y += s.ldY; o1 += sk;)
+#undef OFFSET
+#undef NEAR
+}
+#undef DRR_MINOR_PIECES
+#undef DRR_MINOR_BLOCK
+
+// Whole-ray sums of the pieces, added in piece order.
+struct SlabTotals {
+  float S, g0, c0, h0, g1, c1, h1;
+  __device__ __forceinline__ void add(int slot, const MinorSums& r) {
+    if (slot == 2) {
+      S += r.g;
+    } else if (slot == 0) {
+      g0 += r.g;
+      c0 += r.c;
+      h0 += r.h;
+    } else {
+      g1 += r.g;
+      c1 += r.c;
+      h1 += r.h;
+    }
+  }
+};
+
+// What the ray's end takes from the walk: F in alpha units; with the Jacobian
+// the per-axis crossing sums G = sum w, A = sum w alpha (w = V before - V
+// after, alpha from the entry; A of the dominant axis is not used), and the
+// parts of the clamped end points (Gc, Ac), which belong to no axis.
 struct JacSums {
   float F, G[3], A[3], Gc, Ac;
   int dom;
 };
-
-constexpr float kTieRel = 2.98023223876953125e-7f;  // 1.25 * 2^-22
-constexpr float kTieAbs = 9.765625e-4f;             // 2^-10 high-word units
-
-// Per-ray constants of the Jacobian walk: the slot relabelling (slot 2 is the
-// axis with most crossings), each slot's signed stride and FP32 plane spacing,
-// and the chunk length.  jac_prepare also stores each slot's exact sequence
-// (first crossing, spacing, count) in the lane's shared-memory scratch.
-struct JacRay {
-  int dom, a0, a1;
-  int step[3];
-  float dl[3];
-  int chunk;
+// exact_rays' answer: the sums and the ray's entry in world coordinates, amin
+// and 1 - 2 amin.
+struct ExactRay {
+  JacSums q;
+  float e[3], amin, c;
 };
 
-// State of the Jacobian walk at a chunk boundary.
-struct JacState {
-  unsigned int k0, k1, k2;  // crossings taken per slot
-  unsigned long long O;     // exact position of the last crossing taken (the anchor)
-  int off;                  // voxel after it (padded offset)
-  float v, vprev;           // voxel after and before it
-  bool p0, p1;              // its slot (neither: slot 2 or a clamped entry), whose weight is not yet summed
-};
+// Crossings of an axis (first one at A, spacing D, cnt of them) that precede
+// position pos: those at a smaller position, and with `tie` those at the same one.
+__device__ __forceinline__ int count_before(u64 pos, bool tie, u64 A, u64 D, int cnt, float rd) {
+  if (cnt <= 0 || pos < A) return 0;
+  int n = min(static_cast<int>(fix_to_float(static_cast<long long>(pos - A)) * rd), cnt);
+  while (n < cnt && (fix_at(A, D, static_cast<u32>(n)) < pos || (tie && fix_at(A, D, static_cast<u32>(n)) == pos))) ++n;
+  while (n > 0 && !(fix_at(A, D, static_cast<u32>(n - 1)) < pos || (tie && fix_at(A, D, static_cast<u32>(n - 1)) == pos))) --n;
+  return n;
+}
 
-// One chunk's contribution: the segment sum f (its last segment ending at the
-// exact anchor of the next chunk) and the two slots' weight sums in local
-// positions, with the chunk's anchor as FP32 (Of).
-struct JacChunk {
-  float f, g0, g1, h0, h1, Of;
-};
-
-__device__ __forceinline__ void jac_prepare(const RaySetup& r, JacScratch* ws, JacRay& jr) {
-  const int t = threadIdx.x;
-  int dom = 0;
-  if (r.cnt[1] > r.cnt[dom]) dom = 1;
-  if (r.cnt[2] > r.cnt[dom]) dom = 2;
-  jr.dom = dom;
-  jr.a0 = dom == 0 ? 1 : 0;  // real axis of slot 0
-  jr.a1 = dom == 2 ? 1 : 2;  // real axis of slot 1
-  const int ax_of[3] = {jr.a0, jr.a1, dom};
+// The rays of `mask` (lanes of the warp, each lane's pixel in h, w) in exact
+// crossing order: positions as 64-bit fixed point, ties to the lower axis, after
+// an FP64 clip.  Out of line, for the rays that the slab walk could not order
+// and those whose sum is not finite.  All 32 lanes share one ray's crossings: a
+// crossing's place in the order needs only its position (the other axes'
+// crossings before it are counted), so nothing is serial; one lane walking such
+// a ray alone took ~250 us of dependent gathers, and the kernel waited for it.
+template <int DT>
+__device__ __noinline__ void exact_rays(const VolumeDev& vd, const PoseGeom& pg, u32 mask, int h, int w,
+                                        ExactRay* out) {
+  constexpr u32 kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  for (; mask; mask &= mask - 1u) {
+    const int L = __ffs(static_cast<int>(mask)) - 1;
+    const int hh = __shfl_sync(kAll, h, L), ww = __shfl_sync(kAll, w, L);
+    ExactRay x{};
+    RaySetup r;
+    if (ray_setup(vd, pg, hh, ww, r) > 0) {  // the same for all lanes
+      JacSums& q = x.q;
 #pragma unroll
-  for (int sl = 0; sl < 3; ++sl) {
-    const int a = ax_of[sl];
-    const unsigned long long D = pick3(a, r.D[0], r.D[1], r.D[2]);
-    ws->A0[sl][t] = pick3(a, r.A0[0], r.A0[1], r.A0[2]);
-    ws->D[sl][t] = D;
-    jr.step[sl] = pick3(a, r.step[0], r.step[1], r.step[2]);
-    ws->cnt[sl][t] = pick3(a, r.cnt[0], r.cnt[1], r.cnt[2]);
-    jr.dl[sl] = fix_to_float(static_cast<long long>(D));
-  }
-  jr.chunk = walk_chunk(r.nseg);
-}
-
-// The state before the first crossing: the entry voxel, the entry crossing pending.
-template <int DT>
-__device__ __forceinline__ void jac_start(const VolumeDev& vd, const RaySetup& r, const JacRay& jr, JacState& s) {
-  s.k0 = s.k1 = s.k2 = 0u;
-  s.O = 0ull;
-  s.off = r.off;
-  s.v = gather<DT>(vd, s.off);
-  s.vprev = 0.f;
-  s.p0 = r.ea == jr.a0;
-  s.p1 = r.ea == jr.a1;
-}
-
-// One chunk of n crossings from state s (more: crossings follow the chunk).
-template <int DT>
-__device__ __forceinline__ void jac_chunk(const VolumeDev& vd, const JacRay& jr, JacScratch* ws, JacState& s, int n,
-                                          bool more, JacChunk& out) {
-  const int t = threadIdx.x;
-  const int* step = jr.step;
-  const float* dl = jr.dl;
-  unsigned long long O = s.O;
-  int off = s.off;
-  float v = s.v, vprev = s.vprev;
-  bool p0 = s.p0, p1 = s.p1;
-  ws->c_off[t] = off;
-  ws->c_v[t] = v;
-  ws->c_vprev[t] = vprev;
-  ws->c_pend[t] = p0 ? 0 : (p1 ? 1 : 2);
-  const float x0 = local_pos(fix_at(ws->A0[0][t], ws->D[0][t], s.k0), O);
-  const float y0 = local_pos(fix_at(ws->A0[1][t], ws->D[1][t], s.k1), O);
-  const float z0 = local_pos(fix_at(ws->A0[2][t], ws->D[2][t], s.k2), O);
-  float tx = x0, ty = y0, tz = z0;
-  float lx = 0.f, ly = 0.f, lz = 0.f;
-  // chunk sums in local positions
-  float ac = 0.f, f = 0.f, g0 = 0.f, g1 = 0.f, h0 = 0.f, h1 = 0.f;
-#define DRR_JAC_STEP(an, bx, by)                           \
-  const float an = fminf(fminf(tx, ty), tz);               \
-  const bool bx = tx == an;                                \
-  const bool by = !bx && ty == an;                         \
-  {                                                        \
-    const bool bz = !bx && !by;                            \
-    off += bx ? step[0] : (by ? step[1] : step[2]);        \
-    if (bx) lx += 1.f;                                     \
-    if (by) ly += 1.f;                                     \
-    if (bz) lz += 1.f;                                     \
-    next_xy(tx, ty, lx, ly, dl[0], dl[1], x0, y0);         \
-    tz = fmaf(lz, dl[2], z0);                              \
-  }
-#define DRR_JAC_ACCOUNT()                                  \
-  {                                                        \
-    const float wgt = vprev - v;                           \
-    if (p0) { g0 += wgt; h0 = fmaf(wgt, ac, h0); }         \
-    if (p1) { g1 += wgt; h1 = fmaf(wgt, ac, h1); }         \
-  }
-  // The gathers run two crossings ahead: crossing m+1 (an1, q0/q1, voxel v1
-  // after it) is taken while segment m is summed, and a crossing's weight is
-  // taken once the voxel after it has had one walk step to arrive.  First the
-  // pending crossing at the anchor.
-  DRR_JAC_ACCOUNT()
-  DRR_JAC_STEP(a1st, b1x, b1y)
-  float an1 = a1st;
-  bool q0 = b1x, q1 = b1y;
-  float v1 = gather<DT>(vd, off);
-  float gmin = 3.0e38f;
-#pragma unroll kJacUnroll
-  for (int m = 1; m < n; ++m) {
-    DRR_JAC_STEP(an2, bx, by)
-    const float v2 = gather<DT>(vd, off);
-    const float seg = an1 - ac;
-    gmin = fminf(gmin, seg);
-    f = fmaf(seg, v, f);
-    {  // crossing m, at the end of the segment just summed
-      const float wgt = v - v1;
-      if (q0) { g0 += wgt; h0 = fmaf(wgt, an1, h0); }
-      if (q1) { g1 += wgt; h1 = fmaf(wgt, an1, h1); }
-    }
-    ac = an1;
-    q0 = bx;
-    q1 = by;
-    v = v1;
-    v1 = v2;
-    an1 = an2;
-  }
-  // drain: the segment that ends at the chunk's last crossing, which stays pending
-  {
-    const float seg = an1 - ac;
-    gmin = fminf(gmin, seg);
-    f = fmaf(seg, v, f);
-  }
-  ac = an1;
-  p0 = q0;
-  p1 = q1;
-  vprev = v;
-  v = v1;
-  unsigned int c0 = static_cast<unsigned int>(lx), c1 = static_cast<unsigned int>(ly),
-               c2 = static_cast<unsigned int>(lz);
-  // The float order is exact unless two crossings came within the FP32 error
-  // of the local positions: check the chunk's shortest segment and the gap to
-  // the next crossing after it.
-  const float next = fminf(fminf(tx, ty), tz);
-  if (gmin < fmaf(ac, kTieRel, kTieAbs) || (more && next - ac < fmaf(next, kTieRel, kTieAbs))) {
-    // exact re-walk of the chunk: the next crossing of each slot held as 64-bit
-    // fixed point (all ones once the slot's crossings are used up), the
-    // smallest taken each step (ties to the lower slot)
-    off = ws->c_off[t];
-    v = ws->c_v[t];
-    vprev = ws->c_vprev[t];
-    const int pend = ws->c_pend[t];
-    p0 = pend == 0;
-    p1 = pend == 1;
-    ac = f = g0 = g1 = h0 = h1 = 0.f;
-    c0 = c1 = c2 = 0u;
-    int r0 = ws->cnt[0][t] - static_cast<int>(s.k0), r1 = ws->cnt[1][t] - static_cast<int>(s.k1),
-        r2 = ws->cnt[2][t] - static_cast<int>(s.k2);
-    unsigned long long e0 = r0 > 0 ? fix_at(ws->A0[0][t], ws->D[0][t], s.k0) : ~0ull;
-    unsigned long long e1 = r1 > 0 ? fix_at(ws->A0[1][t], ws->D[1][t], s.k1) : ~0ull;
-    unsigned long long e2 = r2 > 0 ? fix_at(ws->A0[2][t], ws->D[2][t], s.k2) : ~0ull;
-    for (int m = 0; m < n; ++m) {
-      DRR_JAC_ACCOUNT()
-      const bool sx = e0 <= e1 && e0 <= e2;
-      const bool sy = !sx && e1 <= e2;
-      unsigned long long best;
-      if (sx) {
-        best = e0;
-        off += step[0];
-        ++c0;
-        e0 = --r0 > 0 ? e0 + ws->D[0][t] : ~0ull;
-      } else if (sy) {
-        best = e1;
-        off += step[1];
-        ++c1;
-        e1 = --r1 > 0 ? e1 + ws->D[1][t] : ~0ull;
-      } else {
-        best = e2;
-        off += step[2];
-        ++c2;
-        e2 = --r2 > 0 ? e2 + ws->D[2][t] : ~0ull;
+      for (int a = 0; a < 3; ++a) {
+        const double g = fma(static_cast<double>(hh), pg.gh[a], fma(static_cast<double>(ww), pg.gw[a], pg.g00[a]));
+        x.e[a] = fmaf(static_cast<float>(fma(r.amin, g, pg.u0[a])), vd.delta[a],
+                      -0.5f * static_cast<float>(vd.n[a]) * vd.delta[a]);
       }
-      const float an = local_pos(best, O);
-      const float vn = gather<DT>(vd, off);
-      f = fmaf(an - ac, v, f);
-      ac = an;
-      p0 = sx;
-      p1 = sy;
-      vprev = v;
-      v = vn;
+      x.amin = static_cast<float>(r.amin);
+      x.c = static_cast<float>(1.0 - 2.0 * r.amin);
+      if (r.cnt[1] > r.cnt[0]) q.dom = 1;
+      if (r.cnt[2] > max(r.cnt[0], r.cnt[1])) q.dom = 2;
+      float rd[3];
+      u64 first = kFixMax;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        rd[a] = 1.f / fix_to_float(static_cast<long long>(r.D[a]));
+        if (r.cnt[a] > 0) first = min(first, r.A0[a]);
+      }
+      const float vfirst = gather<DT>(vd, r.off);
+      const float vl =
+          gather<DT>(vd, r.off + r.cnt[0] * r.step[0] + r.cnt[1] * r.step[1] + r.cnt[2] * r.step[2]);
+      float F = lane == 0 ? fix_to_float(static_cast<long long>(first)) * vfirst : 0.f;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;
+        float G = 0.f, A = 0.f;
+        for (int k = lane; k < r.cnt[a]; k += 32) {
+          const u64 pos = fix_at(r.A0[a], r.D[a], static_cast<u32>(k));
+          const int nb = count_before(pos, b < a, r.A0[b], r.D[b], r.cnt[b], rd[b]);
+          const int nc = count_before(pos, c < a, r.A0[c], r.D[c], r.cnt[c], rd[c]);
+          const int off = r.off + k * r.step[a] + nb * r.step[b] + nc * r.step[c];
+          const float vb = gather<DT>(vd, off), va = gather<DT>(vd, off + r.step[a]);
+          u64 next = kFixMax;  // the end of the segment after the crossing
+          if (k + 1 < r.cnt[a]) next = min(next, pos + r.D[a]);
+          if (nb < r.cnt[b]) next = min(next, fix_at(r.A0[b], r.D[b], static_cast<u32>(nb)));
+          if (nc < r.cnt[c]) next = min(next, fix_at(r.A0[c], r.D[c], static_cast<u32>(nc)));
+          F = fmaf(fix_to_float(static_cast<long long>(next - pos)), va, F);
+          const float wgt = vb - va;
+          G += wgt;
+          A = fmaf(wgt, fix_to_float(static_cast<long long>(pos)), A);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          G += __shfl_xor_sync(kAll, G, o);
+          A += __shfl_xor_sync(kAll, A, o);
+        }
+        q.G[a] = G;
+        q.A[a] = A;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) F += __shfl_xor_sync(kAll, F, o);
+      q.F = F * r.unit;
+      const float ex = static_cast<float>(kExitUnits);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        if (a == r.ea) q.G[a] -= vfirst;  // entry crossing: weight 0 - V first, at 0
+        if (a == r.xa) {                  // exit crossing: weight V last - 0
+          q.G[a] += vl;
+          q.A[a] = fmaf(vl, ex, q.A[a]);
+        }
+        q.A[a] *= r.unit;
+      }
+      q.Gc = (r.ea < 0 ? -vfirst : 0.f) + (r.xa < 0 ? vl : 0.f);
+      q.Ac = r.xa < 0 ? vl * ex * r.unit : 0.f;
+      const float rest = pick3(q.dom, q.G[1] + q.G[2], q.G[0] + q.G[2], q.G[0] + q.G[1]) + q.Gc;
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        if (a == q.dom) q.G[a] = -rest;  // the sum of all crossing weights is 0
+    }
+    if (lane == L) *out = x;
+  }
+}
+
+// From the pieces' totals to the ray's sums (see the section comment).
+// Called by all 32 lanes of a warp; live: the lane has a ray.
+template <int MODE, int DT>
+__device__ __forceinline__ void slab_finish(const VolumeDev& vd, const PoseGeom& pg, int h, int w, bool live,
+                                            const SlabRay& s, const SlabTotals& T, bool exact,
+                                            Park* park, JacSums& out) {
+  const int t = threadIdx.x;
+  const float v1 = gather<DT>(vd, s.off);
+  const float vl = gather<DT>(vd, s.off + s.cnt[0] * s.step[0] + s.cnt[1] * s.step[1] + s.cnt[2] * s.step[2]);
+  // sum w (1 - f), f the unbiased fraction
+  const float b0 = static_cast<float>(s.t0) * kTwoM32, b1 = static_cast<float>(s.t1) * kTwoM32;
+  const float m0 = fmaf(-kTwoM32, T.c0, fmaf(b0, T.g0, T.g0));
+  const float m1 = fmaf(-kTwoM32, T.c1, fmaf(b1, T.g1, T.g1));
+  const float F = fmaf(-s.rest, vl, fmaf(v1, s.w1, T.S + (m0 + m1)));
+  // a sum that is not finite (an infinite or NaN voxel) is taken segment by segment instead
+  exact = live && (exact || !(fabsf(F) <= 3.0e38f));
+  const u32 mask = __ballot_sync(0xffffffffu, exact);
+  if (mask) {
+    ExactRay x;
+    exact_rays<DT>(vd, pg, mask, h, w, &x);
+    if (exact) {
+      out = x.q;
+      if (MODE != kGeoGrad) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) park->v[kPkE + a][t] = x.e[a];
+      } else {
+        park->v[kPkE][t] = x.c;
+        park->v[kPkE + 1][t] = x.amin;
+      }
+      return;
     }
   }
-#undef DRR_JAC_STEP
-#undef DRR_JAC_ACCOUNT
-  s.k0 += c0;
-  s.k1 += c1;
-  s.k2 += c2;
-  // the chunk's last crossing (the largest one taken) is the next anchor; the
-  // segment that ends there gets its exact end
-  unsigned long long Onew = O;
-  if (s.k0) Onew = max(Onew, fix_at(ws->A0[0][t], ws->D[0][t], s.k0 - 1u));
-  if (s.k1) Onew = max(Onew, fix_at(ws->A0[1][t], ws->D[1][t], s.k1 - 1u));
-  if (s.k2) Onew = max(Onew, fix_at(ws->A0[2][t], ws->D[2][t], s.k2 - 1u));
-  out.f = fmaf(local_pos(Onew, O) - ac, vprev, f);
-  out.g0 = g0;
-  out.g1 = g1;
-  out.h0 = h0;
-  out.h1 = h1;
-  out.Of = fix_to_float(static_cast<long long>(O));
-  s.O = Onew;
-  s.off = off;
-  s.v = v;
-  s.vprev = vprev;
-  s.p0 = p0;
-  s.p1 = p1;
-}
-
-// Running sums of the Jacobian walk over its chunks, in chunk order (chunk sums
-// to absolute positions: alpha = O + local).
-struct JacTotals {
-  float F, G0, G1, A0, A1;
-};
-
-__device__ __forceinline__ void jac_add_chunk(JacTotals& T, const JacChunk& c) {
-  T.F += c.f;
-  T.G0 += c.g0;
-  T.A0 += fmaf(c.Of, c.g0, c.h0);
-  T.G1 += c.g1;
-  T.A1 += fmaf(c.Of, c.g1, c.h1);
-}
-
-// After the last chunk: the last segment to the exit, the last crossing's
-// weight at its absolute position, the exit crossing, and the sums moved back
-// to alpha units and real axes.  Gc: the clamped entry's weight.
-__device__ __forceinline__ void jac_finish(const RaySetup& r, const JacRay& jr, const JacState& s, JacTotals T,
-                                           float Gc, JacSums& out) {
-  float F = fmaf(local_pos(static_cast<unsigned long long>(kExitUnits) << 32, s.O), s.v, T.F);
-  float G0 = T.G0, G1 = T.G1, A0 = T.A0, A1 = T.A1;
-  {
-    const float last = fix_to_float(static_cast<long long>(s.O));
-    const float wgt = s.vprev - s.v;
-    if (s.p0) { G0 += wgt; A0 = fmaf(wgt, last, A0); }
-    if (s.p1) { G1 += wgt; A1 = fmaf(wgt, last, A1); }
-  }
-  // exit crossing: weight V_last - 0 at the exit
-  const float v = s.v;
-  const float ex = static_cast<float>(kExitUnits);
-  float Ac = 0.f;
-  if (r.xa < 0) { Gc += v; Ac = v * ex; }
-  else if (r.xa == jr.a0) { G0 += v; A0 = fmaf(v, ex, A0); }
-  else if (r.xa == jr.a1) { G1 += v; A1 = fmaf(v, ex, A1); }
-  // back to alpha units and real axes (static indices)
-  const float u = r.unit;
-  out.F = F * u;
-  out.dom = jr.dom;
+  out.F = F * s.rg2;
+  float G0 = -T.g0, G1 = -T.g1;
+  float A0 = -fmaf(park->v[kPkRg][t], T.h0, park->v[kPkF0][t] * T.g0);
+  float A1 = -fmaf(park->v[kPkRg + 1][t], T.h1, park->v[kPkF0 + 1][t] * T.g1);
+  const float ex = vl * park->v[kPkSpan][t];
+  // entry crossing: weight 0 - V first at alpha 0; exit crossing: V last - 0 at the span
+  float Gc = 0.f, Ac = 0.f;
+  if (s.ea < 0) Gc -= v1;
+  if (s.ea == s.ax0) G0 -= v1;
+  if (s.ea == s.ax1) G1 -= v1;
+  if (s.xa < 0) { Gc += vl; Ac = ex; }
+  if (s.xa == s.ax0) { G0 += vl; A0 += ex; }
+  if (s.xa == s.ax1) { G1 += vl; A1 += ex; }
+  out.dom = s.ax2;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    out.G[a] = a == jr.a0 ? G0 : (a == jr.a1 ? G1 : -(G0 + G1 + Gc));  // sum of all crossing weights is 0
-    out.A[a] = a == jr.a0 ? A0 * u : (a == jr.a1 ? A1 * u : 0.f);      // the dominant axis is handled through R
+  for (int a = 0; a < 3; ++a) {  // static indices: the arrays stay in registers
+    out.G[a] = a == s.ax0 ? G0 : (a == s.ax1 ? G1 : -(G0 + G1 + Gc));  // sum of all crossing weights is 0
+    out.A[a] = a == s.ax0 ? A0 : (a == s.ax1 ? A1 : 0.f);              // the dominant axis is handled through R
   }
   out.Gc = Gc;
-  out.Ac = Ac * u;
-}
-
-template <int DT>
-__device__ __forceinline__ void walk_jacobian(const VolumeDev& vd, const RaySetup& r, JacScratch* ws,
-                                              JacSums& out) {
-  JacRay jr;
-  jac_prepare(r, ws, jr);
-  JacState s;
-  jac_start<DT>(vd, r, jr, s);
-  const float Gc = r.ea < 0 ? -s.v : 0.f;  // entry clamped at alpha 0: weight -V_first
-  JacTotals T{0.f, 0.f, 0.f, 0.f, 0.f};
-  int remaining = r.nseg - 1;
-  while (remaining > 0) {
-    const int n = min(remaining, jr.chunk);
-    JacChunk c;
-    jac_chunk<DT>(vd, jr, ws, s, n, remaining > n, c);
-    remaining -= n;
-    jac_add_chunk(T, c);
-  }
-  jac_finish(r, jr, s, T, Gc, out);
+  out.Ac = Ac;
 }
 
 // dE/d eta for one ray from the crossing sums (Sec. 2.4 with the voxel lookup
@@ -991,8 +1396,8 @@ __device__ __forceinline__ void walk_jacobian(const VolumeDev& vd, const RaySetu
 // which has no cancellation for rays nearly along that axis.
 //   dE/d eta_j = dE/dt . (dR_j s_c) + dE/dp . (dR_j (p_c - s_c)).
 // gt = dE/dt, gp = dE/dp in world units.
-__device__ __forceinline__ void ray_world_grads(const RaySetup& r, const JacSums& s, float gt[3], float q[3]) {
-  const float L2 = fmaf(r.d[2], r.d[2], fmaf(r.d[1], r.d[1], r.d[0] * r.d[0]));
+__device__ __forceinline__ void ray_world_grads(const float d[3], const JacSums& s, float gt[3], float q[3]) {
+  const float L2 = fmaf(d[2], d[2], fmaf(d[1], d[1], d[0] * d[0]));
   const float L = sqrtf(L2);
   const float F = s.F;
   float R = s.Ac;  // position sums relative to the entry
@@ -1001,17 +1406,17 @@ __device__ __forceinline__ void ray_world_grads(const RaySetup& r, const JacSums
     if (a != s.dom) R += s.A[a];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    if (r.d[a] != 0.f) {
-      const float Ld = L / r.d[a];
+    if (d[a] != 0.f) {
+      const float Ld = L / d[a];
       gt[a] = -s.G[a] * Ld;
       if (a == s.dom) {
         float D = 0.f;
 #pragma unroll
         for (int b = 0; b < 3; ++b)
-          if (b != a) D = fmaf(r.d[b], r.d[b], D);
-        q[a] = (L * R - F * D / L) / r.d[a];
+          if (b != a) D = fmaf(d[b], d[b], D);
+        q[a] = (L * R - F * D / L) / d[a];
       } else {
-        q[a] = r.d[a] * F / L - s.A[a] * Ld;
+        q[a] = d[a] * F / L - s.A[a] * Ld;
       }
     } else {
       gt[a] = 0.f;
@@ -1020,10 +1425,10 @@ __device__ __forceinline__ void ray_world_grads(const RaySetup& r, const JacSums
   }
 }
 
-__device__ __forceinline__ void pose_jacobian(const RaySetup& r, const JacSums& s, const PoseGeom& pg,
+__device__ __forceinline__ void pose_jacobian(const float d[3], const JacSums& s, const PoseGeom& pg,
                                               const float e[3], int h, int w, float scale, float J[6]) {
   float gt[3], q[3];
-  ray_world_grads(r, s, gt, q);
+  ray_world_grads(d, s, gt, q);
   // an angle moves the entry point e by omega_j x (e - t): its term is
   // gt . (omega_j x (e - t)) = omega_j . ((e - t) x gt)
   const float x0 = e[0] - pg.t[0], x1 = e[1] - pg.t[1], x2 = e[2] - pg.t[2];
@@ -1046,12 +1451,11 @@ __device__ __forceinline__ void pose_jacobian(const RaySetup& r, const JacSums& 
 // rho = sdr / 2, p = R (-rho, (w - wc) dw, (h - hc) dh) + t and dE/ds = gt - gp:
 //   dE/dsdr = (dE/ds - dE/dp) . R e_x / 2,
 //   dE/ddh  = (h - hc) dE/dp . R e_z,   dE/ddw = (w - wc) dE/dp . R e_y.
-__device__ __forceinline__ void geometry_jacobian(const RaySetup& r, const JacSums& s, const PoseGeom& pg, int h,
-                                                  int w, float scale, float J[3]) {
+__device__ __forceinline__ void geometry_jacobian(const float d[3], const JacSums& s, const PoseGeom& pg, float am,
+                                                  float c, int h, int w, float scale, float J[3]) {
   float gt[3], q[3];
-  ray_world_grads(r, s, gt, q);
-  // dE/dp = q + amin gt; dE/ds - dE/dp = gt - 2 dE/dp = (1 - 2 amin) gt - 2 q
-  const float am = static_cast<float>(r.amin), c = static_cast<float>(1.0 - 2.0 * r.amin);
+  ray_world_grads(d, s, gt, q);
+  // am = amin, c = 1 - 2 amin; dE/dp = q + amin gt; dE/ds - dE/dp = gt - 2 dE/dp = (1 - 2 amin) gt - 2 q
   float a0 = 0.f, a1 = 0.f, a2 = 0.f;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -1183,69 +1587,80 @@ __device__ __forceinline__ void backproject_tile_ray(const VolumeDev& vd, const 
   RaySetup r{};
   int nseg = 0;
   float gL = 0.f;
-  if (active && ray_setup<false>(vd, pg, h, w, r) > 0) {
+  if (active && ray_setup(vd, pg, h, w, r) > 0) {
     nseg = r.nseg;
     gL = g * sqrtf(fmaf(r.d[2], r.d[2], fmaf(r.d[1], r.d[1], r.d[0] * r.d[0])));
   }
   walk_backproject(vd, r, nseg, gL, gvol, ws, lane);
 }
 
+// The ray's outputs from its sums.
 template <int MODE>
-struct ScratchFor {
-  using type = WalkScratch;
-};
-template <>
-struct ScratchFor<kFwdJac> {
-  using type = JacScratch;
-};
-template <>
-struct ScratchFor<kPoseGrad> {
-  using type = JacScratch;
-};
-template <>
-struct ScratchFor<kGeoGrad> {
-  using type = JacScratch;
-};
+__device__ __forceinline__ void ray_outputs(const VolumeDev& vd, const PoseGeom& pg, int h, int w, const JacSums& q,
+                                            const Park* park, RayResult& res) {
+  const int t = threadIdx.x;
+  const float d[3] = {park->v[kPkD][t], park->v[kPkD + 1][t], park->v[kPkD + 2][t]};
+  res.F = q.F * sqrtf(fmaf(d[2], d[2], fmaf(d[1], d[1], d[0] * d[0]))) * vd.out_scale;
+  if (MODE != kGeoGrad) {
+    const float e[3] = {park->v[kPkE][t], park->v[kPkE + 1][t], park->v[kPkE + 2][t]};
+    pose_jacobian(d, q, pg, e, h, w, vd.out_scale, res.J);
+  } else {
+    geometry_jacobian(d, q, pg, park->v[kPkE + 1][t], park->v[kPkE][t], h, w, vd.out_scale, res.J);
+  }
+}
 
+// Pieces [p0, p1) of the ray's three loops, each piece's sums to sink(p, slot,
+// sums) (slot 2: g alone); true if a pair of crossings in them was too close to
+// order.
+template <int DT, class Sink>
+__device__ __forceinline__ bool walk_pieces(const VolumeDev& vd, const SlabRay& s, const Plan& pl, int p0, int p1,
+                                            Sink sink) {
+  bool near = false;
+  least_loop<DT>(vd, s, pl.slot[1], p0, p1, [&](int p, const MinorSums& r) {
+    near |= r.near < 2u * s.t1;
+    sink(p, 1, r);
+  });
+  middle_loop<DT>(vd, s, pl.slot[0], p0, p1, [&](int p, const MinorSums& r) {
+    near |= r.near < 2u * s.t0;
+    sink(p, 0, r);
+  });
+  dominant_loop<DT>(vd, s, pl.slot[2], p0, p1, [&](int p, float S) { sink(p, 2, MinorSums{S, 0.f, 0.f, 0u}); });
+  return near;
+}
+
+// The rays of one warp tile (all 32 lanes call; a lane outside the detector
+// passes valid = false).
 template <int MODE, int DT>
-__device__ __forceinline__ void trace_ray(const VolumeDev& vd, const PoseGeom& pg, int h, int w, float gscale,
-                                          float* __restrict__ gvol, WalkScratch* ws, RayResult& res) {
+__device__ __forceinline__ void trace_tile(const VolumeDev& vd, const PoseGeom& pg, const GeomFF& gf, int h, int w, bool valid,
+                                           typename ParkFor<MODE>::type* park, RayResult& res) {
   res.F = 0.f;
-  res.nseg = 0;
 #pragma unroll
   for (int k = 0; k < 6; ++k) res.J[k] = 0.f;
-  constexpr bool kJac = MODE == kFwdJac || MODE == kPoseGrad || MODE == kGeoGrad;
-  RaySetup r;
-  float e[3];
-  const int rs = ray_setup<kJac>(vd, pg, h, w, r, e);
-  if (kJac && rs > 0) {  // parked in shared memory until the epilogue
-    JacScratch* js = static_cast<JacScratch*>(ws);
+  if constexpr (MODE == kFwd) {
+    RaySetup r;
+    const int rs = valid ? ray_setup(vd, pg, h, w, r) : 0;
+    if (rs < 0) {
+      res.F = __int_as_float(0x7fffffff);
+    } else if (rs > 0) {
+      const float L = sqrtf(fmaf(r.d[2], r.d[2], fmaf(r.d[1], r.d[1], r.d[0] * r.d[0])));
+      res.F = walk_forward<DT>(vd, r, park) * L * vd.out_scale;
+    }
+  } else {
+    SlabRay s;
+    const int rs = valid ? slab_setup<MODE>(vd, pg, gf, h, w, s, park) : 0;
+    if (rs <= 0) slab_idle(vd, s);
+    bool exact = s.exact;
+    SlabTotals T{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const Plan pl = plan_pieces(s);
+    exact |= walk_pieces<DT>(vd, s, pl, 0, pl.np, [&](int, int slot, const MinorSums& r) { T.add(slot, r); });
+    JacSums q;
+    slab_finish<MODE, DT>(vd, pg, h, w, rs > 0, s, T, exact, park, q);
+    if (rs < 0) {  // non-finite geometry (e.g. a NaN pose): NaN out, no walk
+      res.F = __int_as_float(0x7fffffff);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) js->e[a][threadIdx.x] = e[a];
-  }
-  if (rs < 0) {  // non-finite geometry (e.g. a NaN pose): NaN out, no walk
-    res.F = __int_as_float(0x7fffffff);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) res.J[k] = res.F;
-    return;
-  }
-  if (rs == 0) return;
-  res.nseg = r.nseg;
-  if (MODE == kCount) return;
-  const float L = sqrtf(fmaf(r.d[2], r.d[2], fmaf(r.d[1], r.d[1], r.d[0] * r.d[0])));
-  if (MODE == kFwd) {
-    res.F = walk_forward<DT>(vd, r, ws) * L * vd.out_scale;
-  } else if (MODE == kFwdJac || MODE == kPoseGrad || MODE == kGeoGrad) {
-    JacSums s;
-    walk_jacobian<DT>(vd, r, static_cast<JacScratch*>(ws), s);
-    res.F = s.F * L * vd.out_scale;
-    if (MODE == kGeoGrad) {
-      geometry_jacobian(r, s, pg, h, w, vd.out_scale, res.J);
-      res.J[3] = res.J[4] = res.J[5] = 0.f;
-    } else {
-      const JacScratch* js = static_cast<const JacScratch*>(ws);
-      const float ep[3] = {js->e[0][threadIdx.x], js->e[1][threadIdx.x], js->e[2][threadIdx.x]};
-      pose_jacobian(r, s, pg, ep, h, w, vd.out_scale, res.J);
+      for (int k = 0; k < 6; ++k) res.J[k] = res.F;
+    } else if (rs > 0) {
+      ray_outputs<MODE>(vd, pg, h, w, q, park, res);
     }
   }
 }
@@ -1263,11 +1678,13 @@ __global__ void __launch_bounds__(kThreads, (MODE == kFwdJac || MODE == kPoseGra
                   float* __restrict__ out, float* __restrict__ jac, const float* __restrict__ gin,
                   float* __restrict__ partials, float* __restrict__ gvol) {
   __shared__ PoseGeom spg[kThreads / 32];
-  __shared__ typename ScratchFor<MODE>::type ws;
+  constexpr bool kBp = MODE == kBackproject;
+  constexpr bool kSlab = std::is_same_v<typename ParkFor<MODE>::type, Park>;
+  __shared__ typename ParkFor<MODE>::type ws;
+  __shared__ GeomFF sgf[kSlab ? kThreads / 32 : 1];
   grid_dep_wait();
   grid_dep_release();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr bool kBp = MODE == kBackproject;
   constexpr int TW = kBp ? kBpTileW : kWarpTileW, TH = 32 / TW;
   const int twx = (det.W + TW - 1) / TW;
   const int per_pose = twx * ((det.H + TH - 1) / TH);
@@ -1287,49 +1704,47 @@ __global__ void __launch_bounds__(kThreads, (MODE == kFwdJac || MODE == kPoseGra
       unsigned int* dst = reinterpret_cast<unsigned int*>(&pg);
       for (int i = lane; i < static_cast<int>(sizeof(PoseGeom) / 4); i += 32) dst[i] = src[i];
       __syncwarp();
+      if (kSlab) {
+        geom_ff(pg, sgf[warp]);
+        __syncwarp();
+      }
       cur = b;
     }
     const int ty = tin / twx, tx = tin - ty * twx;
     const int h = ty * TH + lane / TW, w = tx * TW + lane % TW;
     const bool valid = (w < det.W) && (h < det.H);
     const size_t pix = static_cast<size_t>(h) * det.W + w;
-    RayResult r;
-    r.nseg = 0;
     float gsc = 0.f;
     if (valid && (MODE == kPoseGrad || MODE == kGeoGrad || kBp)) gsc = gin[b * npix + pix];
-    if (kBp) {
+    if constexpr (kBp) {
       backproject_tile_ray(vd, pg, h, w, valid && gsc != 0.f, gsc, gvol, &ws, lane);
-      continue;
-    }
-    if (valid) {
-      trace_ray<MODE, DT>(vd, pg, h, w, gsc, gvol, &ws, r);
+    } else if constexpr (MODE == kCount) {
+      RaySetup rs;
+      if (valid) reinterpret_cast<int*>(out)[b * npix + pix] = ray_setup(vd, pg, h, w, rs) > 0 ? rs.nseg : 0;
     } else {
-      r.F = 0.f;
+      RayResult r;
+      trace_tile<MODE, DT>(vd, pg, sgf[kSlab ? warp : 0], h, w, valid, &ws, r);
+      if (MODE == kFwd || MODE == kFwdJac) {
+        if (valid) {
+          out[b * npix + pix] = r.F;
+          if (MODE == kFwdJac) {
 #pragma unroll
-      for (int k = 0; k < 6; ++k) r.J[k] = 0.f;
-    }
-    if (MODE == kCount) {
-      if (valid) reinterpret_cast<int*>(out)[b * npix + pix] = r.nseg;
-    } else if (MODE == kFwd || MODE == kFwdJac) {
-      if (valid) {
-        out[b * npix + pix] = r.F;
-        if (MODE == kFwdJac) {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) jac[(static_cast<size_t>(b) * 6 + k) * npix + pix] = r.J[k];
+            for (int k = 0; k < 6; ++k) jac[(static_cast<size_t>(b) * 6 + k) * npix + pix] = r.J[k];
+          }
         }
-      }
-    } else if (MODE == kPoseGrad || MODE == kGeoGrad) {
-      constexpr int nc = MODE == kPoseGrad ? 6 : 3;  // pose or detector parameters
-      float c[nc];
+      } else {
+        constexpr int nc = MODE == kPoseGrad ? 6 : 3;  // pose or detector parameters
+        float c[nc];
 #pragma unroll
-      for (int k = 0; k < nc; ++k) {
-        c[k] = gsc * r.J[k];
+        for (int k = 0; k < nc; ++k) {
+          c[k] = gsc * r.J[k];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) c[k] += __shfl_xor_sync(0xffffffffu, c[k], o);
-      }
-      if (lane == 0) {
+          for (int o = 16; o > 0; o >>= 1) c[k] += __shfl_xor_sync(0xffffffffu, c[k], o);
+        }
+        if (lane == 0) {
 #pragma unroll
-        for (int k = 0; k < nc; ++k) partials[(static_cast<size_t>(b) * per_pose + tin) * nc + k] = c[k];
+          for (int k = 0; k < nc; ++k) partials[(static_cast<size_t>(b) * per_pose + tin) * nc + k] = c[k];
+        }
       }
     }
   }
@@ -1337,98 +1752,28 @@ __global__ void __launch_bounds__(kThreads, (MODE == kFwdJac || MODE == kPoseGra
 
 // ---------------------------------------------------------------------------
 // Split walk for launches too small to fill the GPU (the fused forward +
-// pose-Jacobian mode): each ray is walked by K lanes, lane j taking the j-th
-// of K runs of whole chunks.  A lane rebuilds the exact walk state at its first
-// chunk boundary, walks its chunks with the same code as the whole-ray walk and
-// parks each chunk's sums in shared memory; the ray's first lane then adds all
-// chunk sums in chunk order and finishes the ray.  Every arithmetic step is the
-// whole-ray walk's, in the same order, so the results are the same bits.
+// pose-Jacobian mode): a block of K warps takes
+// one warp tile (8x4 pixels, pose-major); every warp sets up the tile's 32 rays
+// and sums its share of the loops' pieces, which it parks in shared memory, and
+// the first warp adds each ray's pieces in piece order and finishes the rays.
+// The sums and their order are trace_tile's, so the results are the same bits.
 // ---------------------------------------------------------------------------
-constexpr int kSplitMaxChunks = 32;  // rays with more chunks are not split (longer than ~1950 segments)
-
-// Exact walk state after c crossings in the walk's order (by exact position,
-// ties to the lower slot, which is the order every chunk of the whole-ray walk
-// takes: its tie test sends any chunk whose FP32 order could differ to the
-// exact re-walk).  The crossings of each slot before a position X are counted
-// from the arithmetic sequence (Eq. 3) by one 64-bit division, X is pulled back
-// until at most c crossings precede it, and the rest are taken exactly.
-template <int DT>
-__device__ __forceinline__ void jac_state_at(const VolumeDev& vd, const RaySetup& r, const JacRay& jr,
-                                             const JacScratch* ws, int c, JacState& s) {
-  const int t = threadIdx.x;
-  unsigned long long A[3], D[3];
-  unsigned int cnt[3];
-#pragma unroll
-  for (int sl = 0; sl < 3; ++sl) {
-    A[sl] = ws->A0[sl][t];
-    D[sl] = ws->D[sl][t];
-    cnt[sl] = static_cast<unsigned int>(max(ws->cnt[sl][t], 0));
-  }
-  unsigned int n[3] = {0u, 0u, 0u};
-  const unsigned int total = static_cast<unsigned int>(r.nseg - 1);
-  unsigned long long X = static_cast<unsigned long long>(static_cast<double>(c) / total * 0.98 * kFixScale);
-  for (int it = 0; it < 16; ++it) {
-    unsigned int sum = 0u;
-#pragma unroll
-    for (int sl = 0; sl < 3; ++sl) {
-      n[sl] = (cnt[sl] == 0u || X <= A[sl]) ? 0u
-                                            : static_cast<unsigned int>(min((X - A[sl] - 1ull) / D[sl] + 1ull,
-                                                                            static_cast<unsigned long long>(cnt[sl])));
-      sum += n[sl];
-    }
-    if (sum <= static_cast<unsigned int>(c)) break;
-    X = it < 14 ? X / (sum + 1u) * static_cast<unsigned int>(c) : 0ull;  // the last pass counts from the entry
-  }
-  unsigned long long e[3];
-#pragma unroll
-  for (int sl = 0; sl < 3; ++sl) e[sl] = n[sl] < cnt[sl] ? fix_at(A[sl], D[sl], n[sl]) : ~0ull;
-  for (unsigned int m = n[0] + n[1] + n[2]; m < static_cast<unsigned int>(c); ++m) {
-    const bool sx = e[0] <= e[1] && e[0] <= e[2];
-    const bool sy = !sx && e[1] <= e[2];
-    if (sx) { ++n[0]; e[0] = n[0] < cnt[0] ? e[0] + D[0] : ~0ull; }
-    else if (sy) { ++n[1]; e[1] = n[1] < cnt[1] ? e[1] + D[1] : ~0ull; }
-    else { ++n[2]; e[2] = n[2] < cnt[2] ? e[2] + D[2] : ~0ull; }
-  }
-  // the last crossing taken: the largest position (ties: the higher slot, taken later)
-  unsigned long long O = 0ull;
-  int last = -1;
-#pragma unroll
-  for (int sl = 0; sl < 3; ++sl) {
-    if (n[sl] > 0u) {
-      const unsigned long long q = fix_at(A[sl], D[sl], n[sl] - 1u);
-      if (last < 0 || q >= O) { O = q; last = sl; }
-    }
-  }
-  s.k0 = n[0];
-  s.k1 = n[1];
-  s.k2 = n[2];
-  s.O = O;
-  s.off = r.off + static_cast<int>(n[0]) * jr.step[0] + static_cast<int>(n[1]) * jr.step[1] +
-          static_cast<int>(n[2]) * jr.step[2];
-  s.v = gather<DT>(vd, s.off);
-  s.vprev = gather<DT>(vd, s.off - pick3(last, jr.step[0], jr.step[1], jr.step[2]));
-  s.p0 = last == 0;
-  s.p1 = last == 1;
-}
-
-// Persistent split kernel (mode kFwdJac): a block of K warps claims one warp
-// tile (8x4 pixels, pose-major) at a time; warp j walks the j-th run of chunks
-// of all 32 rays (so a warp's lanes are neighbouring rays, as in the whole-ray
-// kernel, and share cache lines); then the first warp adds each ray's chunk
-// sums in chunk order and finishes the rays.
 template <int DT, int K>
 __global__ void __launch_bounds__(32 * K) siddon_split_kernel(VolumeDev vd, DetDev det, const PoseGeom* __restrict__ pgs,
                                                               int B, unsigned int* __restrict__ counter,
                                                               float* __restrict__ out, float* __restrict__ jac) {
   __shared__ PoseGeom pg;
-  __shared__ JacScratch ws;  // indexed by threadIdx.x (< 32 K)
-  __shared__ JacState fin[32];
-  __shared__ float gcs[32];
+  __shared__ GeomFF gf;
+  __shared__ Park park;  // indexed by threadIdx.x (< 32 K)
+  __shared__ struct {
+    float3 minor[2][32];
+    float S[32];
+  } piece[kPieces];
+  __shared__ unsigned int exact_s[K];
   __shared__ unsigned int tile_s;
-  extern __shared__ JacChunk split_chunks[];  // [kSplitMaxChunks][32]: chunk k of ray i at k * 32 + i
   grid_dep_wait();
   grid_dep_release();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, piece = warp;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int twx = (det.W + kWarpTileW - 1) / kWarpTileW;
   const int per_pose = twx * ((det.H + kWarpTileH - 1) / kWarpTileH);
   const unsigned int total = static_cast<unsigned int>(per_pose) * static_cast<unsigned int>(B);
@@ -1445,58 +1790,54 @@ __global__ void __launch_bounds__(32 * K) siddon_split_kernel(VolumeDev vd, DetD
       const unsigned int* src = reinterpret_cast<const unsigned int*>(pgs + b);
       unsigned int* dst = reinterpret_cast<unsigned int*>(&pg);
       for (int i = threadIdx.x; i < static_cast<int>(sizeof(PoseGeom) / 4); i += 32 * K) dst[i] = src[i];
+      __syncthreads();
+      if (warp == 0) geom_ff(pg, gf);
       cur = b;
     }
     __syncthreads();
     const int ty = tin / twx, tx = tin - ty * twx;
     const int h = ty * kWarpTileH + lane / kWarpTileW, w = tx * kWarpTileW + lane % kWarpTileW;
     const bool valid = (w < det.W) && (h < det.H);
-    RaySetup r;
-    float e[3];
-    const int rs = valid ? ray_setup<true>(vd, pg, h, w, r, e) : 0;
-    JacRay jr;
-    JacState s{};
-    int nch = 0;
-    if (rs > 0) {
-      jac_prepare(r, &ws, jr);
-      const int ncross = r.nseg - 1;
-      nch = (ncross + jr.chunk - 1) / jr.chunk;  // at most kSplitMaxChunks (checked on the host)
-      const int cb = nch * piece / K, ce = nch * (piece + 1) / K;
-      if (cb == 0) {  // the first run, or no crossing at all: from the entry
-        jac_start<DT>(vd, r, jr, s);
-        if (piece == 0) gcs[lane] = r.ea < 0 ? -s.v : 0.f;  // entry clamped at alpha 0: weight -V_first
-      } else if (cb < ce) {
-        jac_state_at<DT>(vd, r, jr, &ws, cb * jr.chunk, s);
-      }
-      for (int k = cb; k < ce; ++k) {
-        const int remaining = ncross - k * jr.chunk;
-        const int n = min(remaining, jr.chunk);
-        jac_chunk<DT>(vd, jr, &ws, s, n, remaining > n, split_chunks[k * 32 + lane]);
-      }
-      // the final state: the last run's (piece K - 1 walks the ray's last
-      // chunk), or piece 0's when the ray has no crossing
-      if (piece == (nch > 0 ? K - 1 : 0)) fin[lane] = s;
-    }
+    SlabRay s;
+    const int rs = valid ? slab_setup<kFwdJac>(vd, pg, gf, h, w, s, &park) : 0;
+    if (rs <= 0) slab_idle(vd, s);
+    bool exact = s.exact;
+    const Plan pl = plan_pieces(s);
+    // this warp's share of the pieces
+    exact |= walk_pieces<DT>(vd, s, pl, pl.np * warp / K, pl.np * (warp + 1) / K,
+                                   [&](int p, int slot, const MinorSums& r) {
+                                     if (slot == 2) piece[p].S[lane] = r.g;
+                                     else piece[p].minor[slot][lane] = make_float3(r.g, r.c, r.h);
+                                   });
+    const unsigned int ex = __ballot_sync(0xffffffffu, exact);
+    if (lane == 0) exact_s[warp] = ex;
     __syncthreads();
-    if (warp == 0 && valid) {
-      const size_t pix = static_cast<size_t>(h) * det.W + w;
-      float F = 0.f, J[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      if (rs < 0) {
-        F = __int_as_float(0x7fffffff);
+    if (warp == 0) {
+      RayResult r;
+      r.F = rs < 0 ? __int_as_float(0x7fffffff) : 0.f;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) J[k] = F;
-      } else if (rs > 0) {
-        JacTotals T{0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int k = 0; k < nch; ++k) jac_add_chunk(T, split_chunks[k * 32 + lane]);
-        JacSums js;
-        jac_finish(r, jr, fin[lane], T, gcs[lane], js);
-        const float L = sqrtf(fmaf(r.d[2], r.d[2], fmaf(r.d[1], r.d[1], r.d[0] * r.d[0])));
-        F = js.F * L * vd.out_scale;
-        pose_jacobian(r, js, pg, e, h, w, vd.out_scale, J);
+      for (int k = 0; k < 6; ++k) r.J[k] = r.F;
+      SlabTotals T{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      for (int p = 0; p < pl.np; ++p) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const float3 q = piece[p].minor[k][lane];
+          T.add(k, MinorSums{q.x, q.y, q.z, 0u});
+        }
+        T.add(2, MinorSums{piece[p].S[lane], 0.f, 0.f, 0u});
       }
-      out[b * npix + pix] = F;
+      unsigned int any = 0u;
 #pragma unroll
-      for (int k = 0; k < 6; ++k) jac[(static_cast<size_t>(b) * 6 + k) * npix + pix] = J[k];
+      for (int k = 0; k < K; ++k) any |= exact_s[k];
+      JacSums q;
+      slab_finish<kFwdJac, DT>(vd, pg, h, w, rs > 0, s, T, (any >> lane) & 1u, &park, q);
+      if (rs > 0) ray_outputs<kFwdJac>(vd, pg, h, w, q, &park, r);
+      if (valid) {
+        const size_t pix = static_cast<size_t>(h) * det.W + w;
+        out[b * npix + pix] = r.F;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) jac[(static_cast<size_t>(b) * 6 + k) * npix + pix] = r.J[k];
+      }
     }
   }
 }
@@ -1726,12 +2067,12 @@ __global__ void __launch_bounds__(32) serve_setup_kernel(const ServeHeader* __re
 }
 
 template <int MODE>
-__device__ __forceinline__ void serve_trace(const VolumeDev& vd, const PoseGeom& pg, int h, int w, float gsc,
-                                            WalkScratch* ws, RayResult& r) {
+__device__ __forceinline__ void serve_trace(const VolumeDev& vd, const PoseGeom& pg, const GeomFF& gf, int h, int w, bool valid,
+                                            typename ParkFor<MODE>::type* park, RayResult& r) {
   switch (vd.dtype) {
-    case kF32: trace_ray<MODE, kF32>(vd, pg, h, w, gsc, nullptr, ws, r); break;
-    case kBF16: trace_ray<MODE, kBF16>(vd, pg, h, w, gsc, nullptr, ws, r); break;
-    default: trace_ray<MODE, kF16>(vd, pg, h, w, gsc, nullptr, ws, r); break;
+    case kF32: trace_tile<MODE, kF32>(vd, pg, gf, h, w, valid, park, r); break;
+    case kBF16: trace_tile<MODE, kBF16>(vd, pg, gf, h, w, valid, park, r); break;
+    default: trace_tile<MODE, kF16>(vd, pg, gf, h, w, valid, park, r); break;
   }
 }
 
@@ -1747,7 +2088,11 @@ __global__ void __launch_bounds__(kThreads, 4) serve_walk_kernel(const ServeHead
                                                                  int* __restrict__ counter) {
   __shared__ PoseGeom spg[kThreads / 32];
   __shared__ ServeRequest sreq[kThreads / 32];
-  __shared__ JacScratch ws;
+  __shared__ GeomFF sgf[kThreads / 32];
+  __shared__ struct {  // apart: at any time a block's warps may walk tiles of both kinds
+    ParkFor<kPoseGrad>::type grad;
+    ParkFor<kFwd>::type fwd;
+  } park;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nreq = hdr->nreq, total = hdr->total_tiles;
   ServeRequest& sr = sreq[warp];
@@ -1780,6 +2125,8 @@ __global__ void __launch_bounds__(kThreads, 4) serve_walk_kernel(const ServeHead
       unsigned int* dst = reinterpret_cast<unsigned int*>(&pg);
       for (int i = lane; i < static_cast<int>(sizeof(PoseGeom) / 4); i += 32) dst[i] = src[i];
       __syncwarp();
+      geom_ff(pg, sgf[warp]);
+      __syncwarp();
       cur_b = b;
     }
     const int twx = (sr.det.W + kWarpTileW - 1) / kWarpTileW;
@@ -1790,19 +2137,14 @@ __global__ void __launch_bounds__(kThreads, 4) serve_walk_kernel(const ServeHead
     const size_t pix = static_cast<size_t>(h) * sr.det.W + w;
     const bool want_grad = sr.grad != nullptr;
     RayResult res;
-    res.F = 0.f;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) res.J[k] = 0.f;
     float gsc = 0.f;
-    if (valid) {
-      if (want_grad) {
-        gsc = sr.grad[b * npix + pix];
-        serve_trace<kPoseGrad>(sr.vd, pg, h, w, gsc, &ws, res);
-      } else {
-        serve_trace<kFwd>(sr.vd, pg, h, w, 0.f, &ws, res);
-      }
-      sr.out[b * npix + pix] = res.F;
+    if (want_grad) {
+      if (valid) gsc = sr.grad[b * npix + pix];
+      serve_trace<kPoseGrad>(sr.vd, pg, sgf[warp], h, w, valid, &park.grad, res);
+    } else {
+      serve_trace<kFwd>(sr.vd, pg, sgf[warp], h, w, valid, &park.fwd, res);
     }
+    if (valid) sr.out[b * npix + pix] = res.F;
     if (want_grad) {  // uniform across the warp: one partial per tile, as a direct render_backward
       float c[6];
 #pragma unroll
@@ -1886,10 +2228,8 @@ int resident_blocks() {
   return v;
 }
 
-// The split kernel with K warps per tile: its dynamic shared memory (the chunk
-// sums of one tile's rays) and the blocks of it the device holds at once
-// (cached per device; 0 if it cannot be configured).
-constexpr size_t kSplitSmem = static_cast<size_t>(kSplitMaxChunks) * 32 * sizeof(JacChunk);
+// The split kernel with K warps per tile: the blocks of it the device holds at
+// once (cached per device).
 template <int DT, int K>
 int split_resident_blocks() {
   constexpr int kMaxDev = 64;
@@ -1900,10 +2240,8 @@ int split_resident_blocks() {
   if (v == 0) {
     int sms = 0, per_sm = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaFuncSetAttribute(siddon_split_kernel<DT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kSplitSmem)) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, siddon_split_kernel<DT, K>, 32 * K, kSplitSmem) !=
-            cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, siddon_split_kernel<DT, K>, 32 * K, 0) !=
+        cudaSuccess) {
       cudaGetLastError();
       v = -1;
     } else {
@@ -1919,22 +2257,16 @@ cudaError_t launch_split(const VolumeDev& vd, const DetDev& det, const PoseGeom*
                          float* out, float* jac, cudaStream_t stream) {
   const int64_t tiles = static_cast<int64_t>(pose_tiles(det)) * B;
   const int grid = static_cast<int>(std::min<int64_t>(tiles, split_resident_blocks<DT, K>()));
-  return launch_pdl_smem(siddon_split_kernel<DT, K>, dim3(grid), dim3(32 * K), kSplitSmem, stream, vd, det, pg, B,
-                         counter, out, jac);
+  return launch_pdl(siddon_split_kernel<DT, K>, dim3(grid), dim3(32 * K), stream, vd, det, pg, B, counter, out,
+                    jac);
 }
 
-// Warps per ray (per warp tile) for a fused forward + Jacobian launch: 8 or 4
-// when the split kernel's resident blocks can take every tile of the launch at
-// once (the whole-ray walk would leave most of the GPU idle, latency-bound on
-// few warps), 1 otherwise.  Rays are split only where every ray fits the split
-// kernel's chunk table (nx + ny + nz <= 61 * kSplitMaxChunks).
-#ifndef DRR_SPLIT
-#define DRR_SPLIT 1
-#endif
+// Warps per ray (per warp tile) for a fused forward + Jacobian launch: 8 or 4 when the split
+// kernel's resident blocks can take every tile of the launch at once (the
+// whole-ray walk would leave most of the GPU idle, latency-bound on few warps),
+// 1 otherwise.
 template <int DT>
-int split_lanes(const VolumeDev& vd, const DetDev& det, int B) {
-  if (!DRR_SPLIT) return 1;
-  if (static_cast<int64_t>(vd.n[0]) + vd.n[1] + vd.n[2] > static_cast<int64_t>(DRR_JAC_LONG) * kSplitMaxChunks) return 1;
+int split_lanes(const DetDev& det, int B) {
   const int64_t tiles = static_cast<int64_t>(pose_tiles(det)) * B;
   if (tiles <= split_resident_blocks<DT, 8>()) return 8;
   if (tiles <= split_resident_blocks<DT, 4>()) return 4;
@@ -1945,7 +2277,7 @@ template <int MODE, int DT>
 cudaError_t launch_siddon_dt(const VolumeDev& vd, const DetDev& det, const PoseGeom* pg, int B, unsigned int* counter,
                              float* out, float* jac, const float* gin, float* partials, float* gvol,
                              cudaStream_t stream, int lanes = 1) {
-  if (MODE == kFwdJac) {
+  if constexpr (MODE == kFwdJac) {
     if (lanes == 8) return launch_split<DT, 8>(vd, det, pg, B, counter, out, jac, stream);
     if (lanes == 4) return launch_split<DT, 4>(vd, det, pg, B, counter, out, jac, stream);
   }
@@ -2115,9 +2447,9 @@ cudaError_t launch_ray_setup(const float* poses, int B, const DetDev& det, float
 
 int render_split_lanes(const VolumeDev& vd, const DetDev& det, int B) {
   switch (vd.dtype) {
-    case kF32: return split_lanes<kF32>(vd, det, B);
-    case kBF16: return split_lanes<kBF16>(vd, det, B);
-    default: return split_lanes<kF16>(vd, det, B);
+    case kF32: return split_lanes<kF32>(det, B);
+    case kBF16: return split_lanes<kBF16>(det, B);
+    default: return split_lanes<kF16>(det, B);
   }
 }
 
