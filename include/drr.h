@@ -212,7 +212,7 @@ drr_status drr_count_segments(drr_volume v, const drr_detector* det, const float
  *  moving_dev, fixed_dev : [B][npix] float32.
  *  loss_dev              : NULL or [B] float32.
  *  grad_dev              : NULL or [B][npix] float32, overwritten with d loss / d moving.
- * Statistics are accumulated in FP64.  Errors: DRR_ERR_INVALID, DRR_ERR_CUDA. */
+ * Statistics are accumulated to FP64 accuracy.  Errors: DRR_ERR_INVALID, DRR_ERR_CUDA. */
 drr_status drr_zncc(const float* moving_dev, const float* fixed_dev, int32_t B, int32_t npix, float eps,
                     float* loss_dev, float* grad_dev, void* cuda_stream);
 

@@ -2,6 +2,10 @@
 // gradient descent on the negative zero-normalised cross-correlation between a
 // moving DRR and a fixed image): the ZNCC loss with its image gradient, and an
 // Adam step on the pose parameters.
+#include <algorithm>
+#include <cstdint>
+
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "drr.h"
@@ -9,71 +13,196 @@
 
 namespace {
 
-constexpr int kZThreads = 512;
+// One thread-block cluster per image pair; block r takes the r-th contiguous
+// share of the pixels.  What bounded one block per pair was FP64 arithmetic (15
+// operations per pixel at 1/64 of the FP32 rate), on one SM per pair.  Per thread
+// the sums now run in FP32 with exact products and exact sums (value + error,
+// Knuth / Dekker), ~2^-47 of a partial sum, and only the threads' partial sums
+// are added in FP64; the image gradient is evaluated the same way from FP64
+// coefficients.  Measured (call with gradient, CUDA events): one 256x256 pair
+// 306 -> 19 us, 64 pairs 308 -> 31 us, 8 pairs of 1024x1024 4400 -> 150 us; 256
+// pairs of 200x200 without gradient 212 -> 68 us, 4096 of them 2770 -> 961 us (two
+// thirds of that the FP64 sums of the partial sums and the closing scalars).
+constexpr int kZThreads = 256;
+constexpr int kZCluster = 8;  // the portable cluster size
+constexpr int kZSums = 5;     // sum I, I^2, F, F^2, I F
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+struct Acc {  // s + e, an unevaluated sum
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float x) {  // exact but for the rounding of e
+    const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)));
+    s = t;
+  }
+  __device__ __forceinline__ void add_product(float x, float y) {
+    const float p = __fmul_rn(x, y);
+    add(p);
+    e = __fadd_rn(e, __fmaf_rn(x, y, -p));
+  }
+};
+
+struct Coefficients {  // d loss / dI = A F + B I + C, each h + l
+  float Ah, Al, Bh, Bl, Ch, Cl;
+};
+
+__device__ __forceinline__ float loss_gradient(const Coefficients& q, float a, float b) {
+  const float p = __fmul_rn(q.Ah, b), r = __fmul_rn(q.Bh, a);
+  Acc t;
+  t.s = p;
+  t.e = __fmaf_rn(q.Al, b, __fmaf_rn(q.Ah, b, -p));
+  t.add(r);
+  t.e = __fadd_rn(t.e, __fmaf_rn(q.Bl, a, __fmaf_rn(q.Bh, a, -r)));
+  t.add(q.Ch);
+  return __fadd_rn(t.s, __fadd_rn(t.e, q.Cl));
 }
 
-// Block-wide sums of n doubles; every thread gets the totals.
-template <int N>
-__device__ __forceinline__ void block_sums(double (&v)[N], double (*sm)[N]) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < N; ++k) v[k] = warp_sum(v[k]);
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < N; ++k) sm[warp][k] = v[k];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    double t = 0.0;
-    for (int q = 0; q < kZThreads / 32; ++q) t += sm[q][k];
-    v[k] = t;
-  }
-  __syncthreads();
+__device__ __forceinline__ void split(double x, float& h, float& l) {
+  h = static_cast<float>(x);
+  l = static_cast<float>(x - static_cast<double>(h));
 }
 
-// One block per image pair.  With population statistics and c = I - mean(I),
-// s = sqrt(mean(c^2)), I^ = c / (s + eps) (same for the fixed image F):
+// Calls f(i, I_i, F_i) for this thread's pixels of [lo, hi), in order; vec: in
+// aligned groups of four (lo and hi are then multiples of 4).
+template <class Fn>
+__device__ __forceinline__ void each_pixel(const float* __restrict__ I, const float* __restrict__ F, int lo, int hi,
+                                           bool vec, Fn f) {
+  if (vec) {
+    for (int i = lo + 4 * static_cast<int>(threadIdx.x); i < hi; i += 4 * kZThreads) {
+      const float4 a = *reinterpret_cast<const float4*>(I + i), b = *reinterpret_cast<const float4*>(F + i);
+      f(i, a.x, b.x);
+      f(i + 1, a.y, b.y);
+      f(i + 2, a.z, b.z);
+      f(i + 3, a.w, b.w);
+    }
+  } else {
+    for (int i = lo + static_cast<int>(threadIdx.x); i < hi; i += kZThreads) f(i, I[i], F[i]);
+  }
+}
+
+// With population statistics and c = I - mean(I), s = sqrt(mean(c^2)),
+// I^ = c / (s + eps) (same for the fixed image F):
 //   zncc = mean(I^ F^),  loss = -zncc,
 //   d zncc / dI_j = (F^_j - zncc c_j / s) / (N (s + eps)).
 // fixed_stride: elements between consecutive fixed images (0: one fixed image for all).
-__global__ void __launch_bounds__(kZThreads) zncc_kernel(const float* __restrict__ moving,
-                                                         const float* __restrict__ fixed, size_t fixed_stride,
-                                                         int npix, float eps, float* __restrict__ loss,
-                                                         float* __restrict__ grad) {
-  __shared__ double sm[kZThreads / 32][5];
-  const size_t base = static_cast<size_t>(blockIdx.x) * npix;
-  const float* I = moving + base;
-  const float* F = fixed + static_cast<size_t>(blockIdx.x) * fixed_stride;
-  double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};  // sum I, sum I^2, sum F, sum F^2, sum I F
-  for (int i = threadIdx.x; i < npix; i += kZThreads) {
-    const double a = I[i], b = F[i];
-    v[0] += a;
-    v[1] += a * a;
-    v[2] += b;
-    v[3] += b * b;
-    v[4] += a * b;
+__global__ void __cluster_dims__(kZCluster, 1, 1) __launch_bounds__(kZThreads)
+    zncc_kernel(const float* __restrict__ moving, const float* __restrict__ fixed, size_t fixed_stride, int npix,
+                float eps, bool vec, float* __restrict__ loss, float* __restrict__ grad) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = static_cast<int>(cluster.block_rank()), pair = static_cast<int>(blockIdx.x / kZCluster);
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  __shared__ double part[kZSums][kZThreads];
+  __shared__ float range[kZThreads / 32];
+  __shared__ double rows[kZCluster][kZSums + 1];  // every block's sums and largest magnitude
+  __shared__ Coefficients coef;
+  __shared__ double coef64[3];
+  const float* I = moving + static_cast<size_t>(pair) * npix;
+  const float* F = fixed + static_cast<size_t>(pair) * fixed_stride;
+  const int unit = vec ? 4 : 1, n = npix / unit;
+  const int lo = static_cast<int>(static_cast<int64_t>(n) * rank / kZCluster) * unit;
+  const int hi = static_cast<int>(static_cast<int64_t>(n) * (rank + 1) / kZCluster) * unit;
+  // products and coefficients of images far from 1 in magnitude would leave the
+  // range of FP32: such images (and images that are not finite) are taken in FP64
+  int wide = 0;
+  for (;; ++wide) {
+    float largest = 0.f;
+    if (!wide) {
+      Acc s[kZSums];
+      float mi = 0.f, mf = 0.f;
+      each_pixel(I, F, lo, hi, vec, [&](int, float a, float b) {
+        s[0].add(a);
+        s[1].add_product(a, a);
+        s[2].add(b);
+        s[3].add_product(b, b);
+        s[4].add_product(a, b);
+        mi = fmaxf(mi, fabsf(a));
+        mf = fmaxf(mf, fabsf(b));
+      });
+      const auto fits = [](float m) { return m == 0.f || (m > 1e-8f && m < 1e10f); };
+      bool ok = true;
+#pragma unroll
+      for (int k = 0; k < kZSums; ++k) {
+        part[k][t] = static_cast<double>(s[k].s) + static_cast<double>(s[k].e);
+        ok = ok && isfinite(s[k].s) && isfinite(s[k].e);
+      }
+      largest = ok && fits(mi) && fits(mf) ? 0.f : 1.f;
+    } else {
+      double s[kZSums] = {0.0, 0.0, 0.0, 0.0, 0.0};
+      each_pixel(I, F, lo, hi, vec, [&](int, float x, float y) {
+        const double a = x, b = y;
+        s[0] += a;
+        s[1] += a * a;
+        s[2] += b;
+        s[3] += b * b;
+        s[4] += a * b;
+      });
+#pragma unroll
+      for (int k = 0; k < kZSums; ++k) part[k][t] = s[k];
+    }
+    const bool any = __any_sync(0xffffffffu, largest != 0.f);
+    if (lane == 0) range[warp] = any ? 1.f : 0.f;
+    __syncthreads();
+    if (warp < kZSums) {  // warp k: the block's sum k, in a fixed order
+      double x = 0.0;
+#pragma unroll
+      for (int q = 0; q < kZThreads / 32; ++q) x += part[warp][32 * q + lane];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      // to every block of the cluster (one of its lanes each)
+      if (lane < kZCluster) cluster.map_shared_rank(&rows[0][0], lane)[rank * (kZSums + 1) + warp] = x;
+    } else if (warp == kZSums && lane < kZCluster) {
+      double x = 0.0;
+#pragma unroll
+      for (int q = 0; q < kZThreads / 32; ++q) x = fmax(x, static_cast<double>(range[q]));
+      cluster.map_shared_rank(&rows[0][0], lane)[rank * (kZSums + 1) + kZSums] = x;
+    }
+    cluster.sync();  // every block's rows are complete in every block
+    bool again = false;
+#pragma unroll
+    for (int r = 0; r < kZCluster; ++r) again = again || rows[r][kZSums] != 0.0;
+    if (wide || !again) break;
+    cluster.sync();  // all blocks have read the rows before they are written again
   }
-  block_sums<5>(v, sm);
-  const double n = static_cast<double>(npix);
-  const double mi = v[0] / n, mf = v[2] / n;
-  const double si = sqrt(fmax(v[1] / n - mi * mi, 0.0)), sf = sqrt(fmax(v[3] / n - mf * mf, 0.0));
-  const double cov = v[4] / n - mi * mf;
-  const double zncc = cov / ((si + eps) * (sf + eps));
-  if (threadIdx.x == 0 && loss) loss[blockIdx.x] = static_cast<float>(-zncc);
+  if (t == 0 && (grad || rank == 0)) {  // every block needs the coefficients, one the loss
+    double v[kZSums];
+#pragma unroll
+    for (int k = 0; k < kZSums; ++k) {
+      double x = 0.0;
+#pragma unroll
+      for (int r = 0; r < kZCluster; ++r) x += rows[r][k];
+      v[k] = x;
+    }
+    const double inv = 1.0 / static_cast<double>(npix);
+    const double mi = v[0] * inv, mf = v[2] * inv;
+    const double si = sqrt(fmax(v[1] * inv - mi * mi, 0.0)), sf = sqrt(fmax(v[3] * inv - mf * mf, 0.0));
+    const double ri = 1.0 / (si + eps), rf = 1.0 / (sf + eps);
+    const double zncc = (v[4] * inv - mi * mf) * ri * rf;
+    if (rank == 0 && loss) loss[pair] = static_cast<float>(-zncc);
+    const double k1 = -inv * ri;  // d loss = -d zncc
+    const double A = k1 * rf, B = si > 0.0 ? -k1 * zncc / si : 0.0;
+    split(A, coef.Ah, coef.Al);
+    split(B, coef.Bh, coef.Bl);
+    split(-(A * mf + B * mi), coef.Ch, coef.Cl);
+    coef64[0] = A;
+    coef64[1] = B;
+    coef64[2] = -(A * mf + B * mi);
+  }
+  cluster.sync();  // no block exits while its rows may still be written; coef is set
   if (!grad) return;
-  const double a_f = 1.0 / (sf + eps);
-  const double k1 = -1.0 / (n * (si + eps));            // d loss = -d zncc
-  const double k2 = si > 0.0 ? zncc / si : 0.0;
-  for (int i = threadIdx.x; i < npix; i += kZThreads) {
-    const double fh = (static_cast<double>(F[i]) - mf) * a_f;
-    const double c = static_cast<double>(I[i]) - mi;
-    grad[base + i] = static_cast<float>(k1 * (fh - k2 * c));
+  const Coefficients q = coef;
+  float* g = grad + static_cast<size_t>(pair) * npix;
+  if (wide) {
+    each_pixel(I, F, lo, hi, vec, [&](int i, float a, float b) {
+      g[i] = static_cast<float>(fma(coef64[0], static_cast<double>(b), fma(coef64[1], static_cast<double>(a), coef64[2])));
+    });
+  } else if (vec) {
+    for (int i = lo + 4 * t; i < hi; i += 4 * kZThreads) {
+      const float4 a = *reinterpret_cast<const float4*>(I + i), b = *reinterpret_cast<const float4*>(F + i);
+      *reinterpret_cast<float4*>(g + i) = make_float4(loss_gradient(q, a.x, b.x), loss_gradient(q, a.y, b.y),
+                                                      loss_gradient(q, a.z, b.z), loss_gradient(q, a.w, b.w));
+    }
+  } else {
+    for (int i = lo + t; i < hi; i += kZThreads) g[i] = loss_gradient(q, I[i], F[i]);
   }
 }
 
@@ -99,7 +228,16 @@ __global__ void adam_kernel(float* __restrict__ params, const float* __restrict_
 
 cudaError_t drr::launch_zncc(const float* moving, const float* fixed, size_t fixed_stride, int B, int npix, float eps,
                              float* loss, float* grad, cudaStream_t stream) {
-  zncc_kernel<<<B, kZThreads, 0, stream>>>(moving, fixed, fixed_stride, npix, eps, loss, grad);
+  const uintptr_t at = reinterpret_cast<uintptr_t>(moving) | reinterpret_cast<uintptr_t>(fixed) |
+                       reinterpret_cast<uintptr_t>(grad);
+  const bool vec = npix % 4 == 0 && fixed_stride % 4 == 0 && at % 16 == 0;
+  constexpr int kMost = 1 << 27;  // pairs per launch (the grid's limit)
+  for (int b = 0; b < B; b += kMost) {
+    const size_t at0 = static_cast<size_t>(b);
+    zncc_kernel<<<kZCluster * std::min(B - b, kMost), kZThreads, 0, stream>>>(
+        moving + at0 * npix, fixed + at0 * fixed_stride, fixed_stride, npix, eps, vec, loss ? loss + at0 : nullptr,
+        grad ? grad + at0 * npix : nullptr);
+  }
   return cudaGetLastError();
 }
 

@@ -102,3 +102,31 @@ def test_registration_step_gradient_full_size(drr):
         G_ref = oracle.pose_grad(ov, odet(det), sub, gE)
         np.testing.assert_allclose(loss.cpu().numpy()[list(picks)], L_ref, atol=1e-5)
         assert grad_err(G[list(picks)], G_ref).max() < GRAD_TOL
+
+
+@pytest.mark.parametrize("npix", [1, 2, 3, 7, 31, 256, 1023, 4096, 40000, 65537])
+@pytest.mark.parametrize("scale,offset", [(1.0, 0.0), (1.0, 1e4), (1e-20, 0.0), (1e20, 0.0)])
+def test_zncc_sizes_and_ranges(drr, npix, scale, offset):
+    # pixel counts around the shares of a cluster's blocks and of their vector loads,
+    # nearly constant images and magnitudes whose squares leave FP32, against NumPy in
+    # FP64: the loss to 2e-7 (its own rounding to FP32 is 6e-8) and the gradient to 1e-6
+    # of its largest entry, widened where the images' variance is a small part of their
+    # mean square (FP64 sums of the squares then lose that much)
+    rng = np.random.default_rng(npix)
+    I = (scale * (offset + rng.uniform(0.5, 3.0, (3, npix)))).astype(np.float32)
+    F = (scale * (offset + rng.uniform(0.5, 3.0, (3, npix)))).astype(np.float32)
+    eps = 1e-8 * scale
+    loss, g = drr.zncc(torch.from_numpy(I).cuda(), torch.from_numpy(F).cuda(), eps)
+    i, f = I.astype(np.float64), F.astype(np.float64)
+    c, d = i - i.mean(1, keepdims=True), f - f.mean(1, keepdims=True)
+    si, sf = np.sqrt((c * c).mean(1, keepdims=True)), np.sqrt((d * d).mean(1, keepdims=True))
+    e = float(np.float32(eps))
+    z = (c * d).mean(1, keepdims=True) / ((si + e) * (sf + e))
+    if npix == 1:  # no variance: only that nothing breaks
+        assert np.isfinite(loss.cpu().numpy()).all()
+        return
+    g_ref = -(d / (sf + e) - z * c / si) / (npix * (si + e))
+    cond = 1e-15 * float(((i * i).mean() + (f * f).mean()) / min((si * si).min(), (sf * sf).min()))
+    assert np.abs(loss.cpu().numpy() + z[:, 0]).max() < 2e-7 + cond
+    if npix > 2:  # (two pixels: the gradient is zero)
+        assert np.abs(g.cpu().numpy() - g_ref).max() < (1e-6 + cond) * np.abs(g_ref).max()
