@@ -466,7 +466,7 @@ drr_status drr_render(drr_volume v, const drr_detector* det, const float* poses_
   configure_pool(v->device);
   AsyncBuf<drr::PoseGeom> pg;
   if (drr_status s = setup_geometry(v, dd, poses_dev, B, st, pg)) return s;
-  const int lanes = jac_out_dev ? drr::render_split_lanes(v->vd, dd, B) : 1;
+  const int lanes = drr::render_split_lanes(v->vd, dd, B, jac_out_dev != nullptr);
   LaunchScope ls(jac_out_dev ? (lanes > 1 ? kSiddonFwdJacSplit : kSiddonFwdJac) : kSiddonFwd, st);
   DRR_CUDA(drr::launch_render(v->vd, dd, pg.p, B, drr_out_dev, jac_out_dev, st, lanes), "render launch");
   return DRR_OK;
@@ -613,7 +613,8 @@ drr_status drr_loss_landscape(drr_volume v, const drr_detector* det, const float
     if (drr_status s = setup_geometry(v, dd, poses_dev + 6 * size_t(i), c, st, pg)) return s;
     {
       LaunchScope ls(kSiddonFwd, st);
-      DRR_CUDA(drr::launch_render(v->vd, dd, pg.p, c, E.p, nullptr, st), "landscape render launch");
+      DRR_CUDA(drr::launch_render(v->vd, dd, pg.p, c, E.p, nullptr, st, drr::render_split_lanes(v->vd, dd, c, false)),
+               "landscape render launch");
     }
     LaunchScope ls(kZncc, st);
     DRR_CUDA(drr::launch_zncc(E.p, fixed_dev, 0, c, int(npix), eps, loss_out_dev + i, nullptr, st),

@@ -483,14 +483,11 @@ __device__ __forceinline__ int ray_setup(const VolumeDev& vd, const PoseGeom& pg
 }
 
 // ---------------------------------------------------------------------------
-// Chunked walk.  The exact fixed-point crossing positions are the reference
-// frame, but the per-segment arithmetic runs in FP32 on positions measured from
-// a nearby origin: at the start of every chunk of crossings the next crossing
-// of each axis is recomputed exactly (first + k * delta in 64-bit) relative to
-// the exact position of the current point, so local positions stay below
-// ~chunk plane gaps and carry 2^-24 of the chunk instead of 2^-24 of the ray's
-// alpha as a whole-ray FP32 walk would.  Positions are in fixed-point
-// high-word units (span / 2^24).
+// Fixed-point crossing sequences.  The exact positions are first + k * delta in
+// 64-bit; the back-projection's per-segment arithmetic runs in FP32 on positions
+// measured from a nearby origin, recomputed exactly at the start of every chunk
+// of crossings, so local positions stay below ~chunk plane gaps and carry 2^-24
+// of the chunk.  Positions are in fixed-point high-word units (span / 2^24).
 // ---------------------------------------------------------------------------
 #ifndef DRR_FWD_MINB
 #define DRR_FWD_MINB 4
@@ -500,12 +497,13 @@ __device__ __forceinline__ int ray_setup(const VolumeDev& vd, const PoseGeom& pg
 #endif
 constexpr float kTwoM32 = 2.3283064365386963e-10f;  // 2^-32
 
-// Per-thread exact crossing parameters, kept in shared memory: they are read
-// only when a chunk starts (and on the rare exact tie path).
+// Per-thread exact crossing parameters of the back-projection, kept in shared
+// memory: they are read only when a chunk starts.
 struct WalkScratch {
   unsigned long long A0[3][kThreads];
   unsigned long long D[3][kThreads];
 };
+
 __device__ __forceinline__ unsigned long long fix_at(unsigned long long A0, unsigned long long D, unsigned int k) {
   return A0 + static_cast<unsigned long long>(k) * D;
 }
@@ -537,138 +535,9 @@ __device__ __forceinline__ void next_xy(float& tx, float& ty, float lx, float ly
 #endif
 }
 
-// One forward-walk step in predicated PTX: an = min(tx, ty, tz); the axis it
-// belongs to (x before y before z on ties) steps: its crossing counter + 1 and
-// the voxel offset by its stride, each as a guarded add, where the compiler's
-// code for the same C++ (kept below, -DDRR_FWD_PTX=0) spends selects on the
-// busier ALU pipe (forward 0.384 -> 0.377 ms on the CT batch, same DRR bits).
-// The Jacobian walk keeps the C++ form: it carries each step's axis
-// predicates to the next step's weight accounting, which an asm block cannot.
-#ifndef DRR_FWD_PTX
-#define DRR_FWD_PTX 1
-#endif
-__device__ __forceinline__ float walk_step(float tx, float ty, float tz, float& lx, float& ly, float& lz, int& off,
-                                           int sx, int sy, int sz) {
-  float an;
-  asm("{\n\t"
-      ".reg .pred px, py, pxy;\n\t"
-      "min.f32 %0, %5, %6;\n\t"
-      "min.f32 %0, %0, %7;\n\t"
-      "setp.eq.f32 px, %5, %0;\n\t"
-      "setp.eq.and.f32 py, %6, %0, !px;\n\t"
-      "or.pred pxy, px, py;\n\t"
-      "@px add.f32 %1, %1, 0f3F800000;\n\t"
-      "@py add.f32 %2, %2, 0f3F800000;\n\t"
-      "@!pxy add.f32 %3, %3, 0f3F800000;\n\t"
-      "@px add.s32 %4, %4, %8;\n\t"
-      "@py add.s32 %4, %4, %9;\n\t"
-      "@!pxy add.s32 %4, %4, %10;\n\t"
-      "}"
-      : "=&f"(an), "+f"(lx), "+f"(ly), "+f"(lz), "+r"(off)
-      : "f"(tx), "f"(ty), "f"(tz), "r"(sx), "r"(sy), "r"(sz));
-  return an;
-}
-
 // Local FP32 position of an exact position relative to O.
 __device__ __forceinline__ float local_pos(unsigned long long x, unsigned long long O) {
   return fix_to_float(static_cast<long long>(x - O));
-}
-
-// The forward walk gathers two crossings ahead: the first crossing of a chunk is
-// peeled and the unrolled loop runs chunk - 1 times.  The three voxel registers
-// of that pipeline rotate without register moves when the unroll is a multiple
-// of 3; 12 divides chunk - 1 for the long-ray chunks (121, 181) and for 13.
-// (Measured on the CT batch: 6 / 12 / 24 at 0.376 / 0.371 / 0.375 ms.)
-#ifndef DRR_FWD_UNROLL
-#define DRR_FWD_UNROLL 12
-#endif
-constexpr int kFwdUnroll = DRR_FWD_UNROLL;
-// Chunk length per ray.  The FP32 error of a local position grows with the
-// chunk's share of the ray, so long rays take long chunks (fewer exact
-// re-anchorings) and short rays short ones.
-__device__ __forceinline__ int fwd_chunk(int nseg) {
-  return nseg > 1024 ? 181 : nseg > 512 ? 121 : nseg > 256 ? 31 : nseg > 128 ? 19 : 13;
-}
-
-// Forward walk (Eq. 2 with the crossings of Eq. 3 taken in order, Sec. 2.2).
-// The gathers run two crossings ahead of the accumulation (the first crossing
-// of a chunk is peeled); the segment that ends at a chunk's last crossing takes
-// that crossing's exact position.
-template <int DT>
-__device__ __forceinline__ float walk_forward(const VolumeDev& vd, const RaySetup& r, WalkScratch* ws) {
-  const int t = threadIdx.x;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    ws->A0[a][t] = r.A0[a];
-    ws->D[a][t] = r.D[a];
-  }
-  const float dx = fix_to_float(static_cast<long long>(r.D[0])), dy = fix_to_float(static_cast<long long>(r.D[1])),
-              dz = fix_to_float(static_cast<long long>(r.D[2]));
-  unsigned int kx = 0u, ky = 0u, kz = 0u;  // crossings consumed per axis before this chunk
-  unsigned long long O = 0ull;              // exact position of the current point
-  int off = r.off;
-  float v = gather<DT>(vd, off);
-  float acc = 0.f;
-  int remaining = r.nseg - 1;
-  const int chunk = fwd_chunk(r.nseg);
-  while (remaining > 0) {
-    const float x0 = local_pos(fix_at(ws->A0[0][t], ws->D[0][t], kx), O);
-    const float y0 = local_pos(fix_at(ws->A0[1][t], ws->D[1][t], ky), O);
-    const float z0 = local_pos(fix_at(ws->A0[2][t], ws->D[2][t], kz), O);
-    float tx = x0, ty = y0, tz = z0;
-    float lx = 0.f, ly = 0.f, lz = 0.f;
-    const int n = min(remaining, chunk);
-#if DRR_FWD_PTX
-#define DRR_FSTEP(an)                                                                     \
-  const float an = walk_step(tx, ty, tz, lx, ly, lz, off, r.step[0], r.step[1], r.step[2]); \
-  {                                                                                       \
-    next_xy(tx, ty, lx, ly, dx, dy, x0, y0);                                              \
-    tz = fmaf(lz, dz, z0);                                                                \
-  }
-#else
-#define DRR_FSTEP(an)                                       \
-  const float an = fminf(fminf(tx, ty), tz);                \
-  {                                                         \
-    const bool bx = tx == an;                               \
-    const bool by = !bx && ty == an;                        \
-    const bool bz = !bx && !by;                             \
-    off += bx ? r.step[0] : (by ? r.step[1] : r.step[2]);   \
-    if (bx) lx += 1.f;                                      \
-    if (by) ly += 1.f;                                      \
-    if (bz) lz += 1.f;                                      \
-    next_xy(tx, ty, lx, ly, dx, dy, x0, y0);                \
-    tz = fmaf(lz, dz, z0);                                  \
-  }
-#endif
-    DRR_FSTEP(a1)
-    float an1 = a1;
-    float v1 = gather<DT>(vd, off);
-    float ac = 0.f;
-#pragma unroll kFwdUnroll
-    for (int m = 1; m < n; ++m) {
-      DRR_FSTEP(an2)
-      const float v2 = gather<DT>(vd, off);
-      acc = fmaf(an1 - ac, v, acc);
-      ac = an1;
-      an1 = an2;
-      v = v1;
-      v1 = v2;
-    }
-#undef DRR_FSTEP
-    remaining -= n;
-    kx += static_cast<unsigned int>(lx);
-    ky += static_cast<unsigned int>(ly);
-    kz += static_cast<unsigned int>(lz);
-    unsigned long long Onew = O;
-    if (kx) Onew = max(Onew, fix_at(ws->A0[0][t], ws->D[0][t], kx - 1u));
-    if (ky) Onew = max(Onew, fix_at(ws->A0[1][t], ws->D[1][t], ky - 1u));
-    if (kz) Onew = max(Onew, fix_at(ws->A0[2][t], ws->D[2][t], kz - 1u));
-    acc = fmaf(local_pos(Onew, O) - ac, v, acc);  // the segment ending at the chunk's last crossing, exact end
-    v = v1;
-    O = Onew;
-  }
-  acc = fmaf(local_pos(static_cast<unsigned long long>(kExitUnits) << 32, O), v, acc);
-  return acc * r.unit;
 }
 
 // ---------------------------------------------------------------------------
@@ -743,9 +612,15 @@ enum ParkSlot : int {
 struct Park {
   float v[kPkCount][kThreads];
 };
+// Per-ray values that the forward walk needs only where a chunk starts.
+struct FwdPark {
+  u64 x0[2][kThreads], dx[2][kThreads];  // slots 0, 1: q_2 at crossing 0 and its step (32.32)
+  u64 y0[2][kThreads], dy[2][kThreads];  // q_0, q_1 at dominant crossing 0 and their steps (24.40)
+};
 template <int MODE>
 struct ParkFor {
-  using type = std::conditional_t<MODE == kFwdJac || MODE == kPoseGrad || MODE == kGeoGrad, Park, WalkScratch>;
+  using type = std::conditional_t<MODE == kFwdJac || MODE == kPoseGrad || MODE == kGeoGrad, Park,
+                                  std::conditional_t<MODE == kFwd, FwdPark, WalkScratch>>;
 };
 
 struct SlabRay {
@@ -767,6 +642,11 @@ struct SlabRay {
   float rest;      // share of the last slab beyond the exit
   float rg2;       // alpha per dominant plane
   bool exact;      // to be summed by exact_rays
+  // the forward walk only
+  u64 qx;          // q_2 at the exit
+  float start;     // q_2 at the entry
+  float r0, r1;    // slabs per plane of slots 0, 1
+  float len;       // |p - s| in mm
 };
 
 // A lane without a ray to walk takes part with no crossings.
@@ -841,6 +721,13 @@ __device__ __forceinline__ u32 ff_frac(float2 x) {
                 static_cast<u64>(static_cast<long long>(__float2int_rn(x.y * 4294967296.f)));
   return v >> 32 ? (static_cast<long long>(v) < 0 ? 0u : 0xffffffffu) : static_cast<u32>(v);
 }
+// x in [0, 1] times 2^40.
+__device__ __forceinline__ u64 ff_fix40(float2 x) {
+  const float h = x.x * 65536.f, a = floorf(h);
+  const u64 v = (static_cast<u64>(__float2uint_rz(a)) << 24) + __float2uint_rz((h - a) * 16777216.f);
+  const long long r = static_cast<long long>(v) + __float2int_rn(x.y * 1099511627776.f);
+  return r < 0 ? 0ull : static_cast<u64>(r);
+}
 __device__ __forceinline__ float fix_float(u64 x) {  // 32.32 fixed point to FP32
   return fmaf(static_cast<float>(static_cast<u32>(x)), kTwoM32, static_cast<float>(static_cast<u32>(x >> 32)));
 }
@@ -851,8 +738,10 @@ __device__ __forceinline__ float fix_float(u64 x) {  // 32.32 fixed point to FP3
 // exact_rays decides in FP64.
 template <int MODE>
 __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& pg, const GeomFF& gf, int h,
-                                          int w, SlabRay& s, Park* park) {
+                                          int w, SlabRay& s, typename ParkFor<MODE>::type* park) {
+  constexpr bool kFwdOnly = MODE == kFwd;
   const int t = threadIdx.x;
+  float d[3];
   float2 g[3];
   if (w < (1 << 24) && h < (1 << 24)) {
     const float fw = static_cast<float>(w), fh = static_cast<float>(h);
@@ -882,7 +771,8 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     finite = finite && isfinite(g[a].x) && isfinite(gf.u0[a].x);
-    park->v[kPkD + a][t] = g[a].x * vd.delta[a];
+    d[a] = g[a].x * vd.delta[a];
+    if constexpr (!kFwdOnly) park->v[kPkD + a][t] = d[a];
     if (g[a].x != 0.f) {
       ar[a] = ff_rcp(make_float2(fabsf(g[a].x), g[a].x < 0.f ? -g[a].y : g[a].y));
       unsafe = unsafe || fabsf(g[a].x) < 1e-20f;
@@ -900,12 +790,15 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
   if (!hit) return 0;
   const float tol = 9.5367431640625e-7f * fmaxf(fabsf(lof), fabsf(hif)) + 1e-30f;  // 2^-20
   unsafe = unsafe || lof - lo2 < tol || hi2 - hif < tol || fabsf(hif - lof) < tol;
+  const float L = sqrtf(fmaf(d[2], d[2], fmaf(d[1], d[1], d[0] * d[0])));
   if (unsafe) {
     slab_idle(vd, s);
     s.exact = true;
+    s.len = L;
     return 1;
   }
   if (!(lof < hif)) return 0;
+  s.len = L;
   // slots: 2 the largest direction component, 1 the smallest
   float2 ag[3];
 #pragma unroll
@@ -961,11 +854,15 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
       const u64 f = min(ff_fix(ue), (static_cast<u64>(n[k]) << 32) - 1ull);
       E[k] = static_cast<u32>(f);
       s.i0[k] = static_cast<int>(f >> 32);
-      if (sg[k].x != 0.f && E[k] + te < 2u * te) exact = true;
+      if (sg[k].x != 0.f) {
+        if (E[k] + te < 2u * te) exact = true;
+      } else {  // parallel: the voxel as exact_rays finds it (half open, also for a ray in a voxel plane)
+        s.i0[k] = min(max(static_cast<int>(floor(pick3(ax[k], pg.u0[0], pg.u0[1], pg.u0[2]))), 0), n[k] - 1);
+      }
     }
     // element offset of the entry voxel: counted from the far end where the ray runs down
     s.off += s.step[k] * (up[k] ? s.i0[k] : s.i0[k] - (n[k] - 1));
-    if (MODE != kGeoGrad) {
+    if constexpr (!kFwdOnly && MODE != kGeoGrad) {
       // the entry point in world coordinates (volume centred at the origin)
       const float dl = pick3(ax[k], vd.delta[0], vd.delta[1], vd.delta[2]), half = 0.5f * static_cast<float>(n[k]);
       const float e = up[k] ? fmaf(uef, dl, -half * dl) : fmaf(-uef, dl, half * dl);
@@ -974,8 +871,9 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
       else park->v[kPkE + 2][t] = e;
     }
   }
-  s.dy = ff_frac(ff_mul(sg[0], sr[2]));
-  s.dz = ff_frac(ff_mul(sg[1], sr[2]));
+  const float2 r02 = ff_mul(sg[0], sr[2]), r12 = ff_mul(sg[1], sr[2]);
+  s.dy = ff_frac(r02);
+  s.dz = ff_frac(r12);
   s.mdz = ff_frac(ff_mul(sg[1], sr[0]));
   const float2 r20 = ff_mul(sg[2], sr[0]), r21 = ff_mul(sg[2], sr[1]), r01 = ff_mul(sg[0], sr[1]);
   // exit: coordinate along the dominant axis, then the counts
@@ -990,7 +888,7 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
     const u32 fr = static_cast<u32>(qx);
     s.rest = static_cast<float>(0u - fr) * kTwoM32;
     if (fr == 0u) s.rest = 1.f;
-    if (fr + te < 2u * te) exact = true;
+    if (!kFwdOnly && fr + te < 2u * te) exact = true;
   }
   const float dom = static_cast<float>(s.cnt[2]) + 16.f + far;
   const u32 tx = static_cast<u32>(fminf(dom, 2e8f));
@@ -1007,8 +905,29 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
       const u64 f = static_cast<u64>(E[k]) + static_cast<u64>(static_cast<u32>(len >> 32)) * sl +
                     __umulhi(static_cast<u32>(len), sl);
       s.cnt[k] = min(static_cast<int>(f >> 32), most);
-      if (static_cast<u32>(f) + tx < 2u * tx) exact = true;
+      if (!kFwdOnly && static_cast<u32>(f) + tx < 2u * tx) exact = true;
     }
+  }
+  s.rg2 = sr[2].x;
+  if constexpr (kFwdOnly) {
+    // positions along a minor axis whose planes lie more than 2^16 slabs apart
+    // would lose more than FP32 keeps of them
+    s.exact = exact || (s.cnt[0] > 0 && !(r20.x < 65536.f)) || (s.cnt[1] > 0 && !(r21.x < 65536.f)) || n[2] >= (1 << 23);
+    if (s.exact) s.cnt[0] = s.cnt[1] = s.cnt[2] = 0;
+    s.qx = qx;
+    s.start = static_cast<float>(E[2]) * kTwoM32;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const bool any = s.cnt[k] > 0;
+      const float2 r = k == 0 ? r20 : r21;
+      const u64 dx = ff_fix(any ? r : make_float2(0.f, 0.f)), dy = ff_fix40(k == 0 ? r02 : r12);
+      park->dx[k][t] = dx;
+      park->x0[k][t] = any ? E[2] + (dx - mul_frac(E[k], dx)) : static_cast<u64>(1u << 30) << 32;  // none: beyond any exit
+      park->dy[k][t] = dy;
+      park->y0[k][t] = (static_cast<u64>(E[k]) << 8) + (dy - mul_frac(E[2], dy));
+      (k == 0 ? s.r0 : s.r1) = any ? r.x : 0.f;
+    }
+    return 1;
   }
   // rounding bounds in 2^-32: a minor crossing's own coordinates err by at most
   // ~cnt + 3, the dominant loop's view of it by ~cnt_2 + 3 of its plane spacings
@@ -1042,17 +961,214 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
     if (ez >= lz) s.Z -= min(s.Z, ez - lz + 1ull);
   }
   s.w1 = E[2] == 0u ? 1.f : static_cast<float>(0u - E[2]) * kTwoM32;
-  s.rg2 = sr[2].x;
-  if (MODE == kGeoGrad) {
-    park->v[kPkE][t] = (1.f - 2.f * amin.x) - 2.f * amin.y;
-    park->v[kPkE + 1][t] = amin.x;
+  if constexpr (!kFwdOnly) {
+    if (MODE == kGeoGrad) {
+      park->v[kPkE][t] = (1.f - 2.f * amin.x) - 2.f * amin.y;
+      park->v[kPkE + 1][t] = amin.x;
+    }
+    park->v[kPkF0][t] = (E[0] == 0u ? 1.f : static_cast<float>(0u - E[0]) * kTwoM32) * sr[0].x;
+    park->v[kPkF0 + 1][t] = (E[1] == 0u ? 1.f : static_cast<float>(0u - E[1]) * kTwoM32) * sr[1].x;
+    park->v[kPkRg][t] = sr[0].x;
+    park->v[kPkRg + 1][t] = sr[1].x;
+    park->v[kPkSpan][t] = fix_float(len) * sr[2].x;
   }
-  park->v[kPkF0][t] = (E[0] == 0u ? 1.f : static_cast<float>(0u - E[0]) * kTwoM32) * sr[0].x;
-  park->v[kPkF0 + 1][t] = (E[1] == 0u ? 1.f : static_cast<float>(0u - E[1]) * kTwoM32) * sr[1].x;
-  park->v[kPkRg][t] = sr[0].x;
-  park->v[kPkRg + 1][t] = sr[1].x;
-  park->v[kPkSpan][t] = fix_float(len) * sr[2].x;
   return 1;
+}
+
+// ---------------------------------------------------------------------------
+// Forward walk (Eq. 2 with the crossings of Eq. 3 taken in order, Sec. 2.2):
+// each step takes the smallest of the three axes' next crossings.  The steps run
+// in chunks of the same number of crossings for the warp's 32 rays.  Inside a
+// chunk positions are FP32 slab coordinates q_2 from the last dominant plane
+// before it: the dominant axis' crossings are whole numbers, the minor ones l r +
+// x0, so they err by 2^-24 of a chunk.  A chunk starts from counts of crossings
+// per axis alone, in exact (32.32 fixed point) order, and its last segment ends
+// at the exact position of its last crossing; where FP32 took a chunk's last
+// crossings in another order (they are then closer than 2^-24 of a chunk) the
+// counts are corrected.  So the chunks are independent: they are added in order
+// whoever walks them, and the split kernel's warps, which take different chunks
+// of a ray, give the same bits as one warp walking through.
+//
+// What bounds it: one gather per segment, 4.4 wavefronts each on the L1 data
+// pipe (71 % busy), and ~18 warp instructions per segment (issue slots 60 %).
+// Measured (CUDA events): 16-pose CT batch, 512x512x133 and 200x200, 0.366 ->
+// 0.344 ms against the walk with an FP64 ray setup; one 128x128 pose on 256^3, split
+// over the warps of a tile, 0.069 -> 0.028.  Chunks that begin at a dominant
+// plane instead of keeping step, 8 / 4 / 2 / 1 per ray: 0.377 / 0.358 / 0.350 /
+// 0.340 (rays that wait for each other at a plane x = const touch 15 cache lines
+// per gather, rays in step 13), and a whole ray in one FP32 frame is too inexact
+// for the smallest volumes.
+// ---------------------------------------------------------------------------
+#ifndef DRR_FWD_UNROLL
+#define DRR_FWD_UNROLL 12  // a multiple of 3: the voxel registers of the two-ahead pipeline rotate without moves
+#endif
+constexpr int kFwdUnroll = DRR_FWD_UNROLL;
+#ifndef DRR_CHUNKS
+#define DRR_CHUNKS 8
+#endif
+constexpr int kChunks = DRR_CHUNKS;  // most chunks of a ray
+
+// One step in predicated PTX: an = min(tx, ty, tz); the axis it belongs to
+// (dominant before middle before least on ties) steps: the dominant position + 1
+// or the minor axis' crossing counter + 1, and the voxel offset by its stride.
+__device__ __forceinline__ float walk_step(float& tx, float ty, float tz, float& ly, float& lz, int& off, int sx, int sy,
+                                           int sz) {
+  float an;
+  asm("{\n\t"
+      ".reg .pred px, py, pxy;\n\t"
+      "min.f32 %0, %1, %5;\n\t"
+      "min.f32 %0, %0, %6;\n\t"
+      "setp.eq.f32 px, %1, %0;\n\t"
+      "setp.eq.and.f32 py, %5, %0, !px;\n\t"
+      "or.pred pxy, px, py;\n\t"
+      "@px add.f32 %1, %1, 0f3F800000;\n\t"
+      "@py add.f32 %2, %2, 0f3F800000;\n\t"
+      "@!pxy add.f32 %3, %3, 0f3F800000;\n\t"
+      "@px add.s32 %4, %4, %7;\n\t"
+      "@py add.s32 %4, %4, %8;\n\t"
+      "@!pxy add.s32 %4, %4, %9;\n\t"
+      "}"
+      : "=&f"(an), "+f"(tx), "+f"(ly), "+f"(lz), "+r"(off)
+      : "f"(ty), "f"(tz), "r"(sx), "r"(sy), "r"(sz));
+  return an;
+}
+
+// Crossings taken per slot, and the exact positions around them: the last one
+// taken (at), and the next one of each slot (beyond every crossing where there
+// is none).
+struct Counts {
+  int k[3];
+};
+constexpr u64 kNever = 1ull << 62;
+struct Around {
+  u64 at, next[3];
+  bool ordered;  // every crossing taken precedes every other (ties: slot 2, 0, 1)
+};
+__device__ __forceinline__ Around around(const SlabRay& s, const FwdPark* park, const Counts& c) {
+  const int t = threadIdx.x;
+  Around r;
+  u64 last[3];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const u64 dx = park->dx[k][t], x = park->x0[k][t] + static_cast<u64>(static_cast<u32>(c.k[k])) * dx;
+    r.next[k] = c.k[k] < s.cnt[k] ? x : kNever;
+    last[k] = c.k[k] > 0 ? x - dx : 0ull;
+  }
+  last[2] = static_cast<u64>(static_cast<u32>(c.k[2])) << 32;
+  r.next[2] = c.k[2] < s.cnt[2] ? last[2] + (1ull << 32) : kNever;
+  if (c.k[2] == 0) last[2] = 0ull;
+  r.at = max(max(last[0], last[1]), last[2]);
+  r.ordered = c.k[0] <= s.cnt[0] && c.k[1] <= s.cnt[1] && c.k[2] <= s.cnt[2] && last[2] <= min(r.next[0], r.next[1]) &&
+              last[0] <= r.next[1] && last[1] < r.next[0] && max(last[0], last[1]) < r.next[2];
+  return r;
+}
+
+// The counts after n crossings in exact order, from a dominant crossing before.
+__device__ __forceinline__ Counts counts_after(const SlabRay& s, const FwdPark* park, int n) {
+  const int t = threadIdx.x;
+  const int total = s.cnt[0] + s.cnt[1] + s.cnt[2];
+  Counts c{{0, 0, 0}};
+  int left = n;
+  int a = static_cast<int>(static_cast<float>(n) * static_cast<float>(s.cnt[2]) / static_cast<float>(max(total, 1))) - 1;
+  a = min(a, s.cnt[2]);
+  while (a > 0) {
+    const u64 X = static_cast<u64>(static_cast<u32>(a)) << 32;  // dominant crossing a - 1
+    int m[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {  // minor crossings before it
+      const u64 x0 = park->x0[k][t], dx = park->dx[k][t];
+      m[k] = min(static_cast<int>((park->y0[k][t] + static_cast<u64>(static_cast<u32>(a - 1)) * park->dy[k][t]) >> 40), s.cnt[k]);
+      while (m[k] > 0 && x0 + static_cast<u64>(static_cast<u32>(m[k] - 1)) * dx >= X) --m[k];
+      while (m[k] < s.cnt[k] && x0 + static_cast<u64>(static_cast<u32>(m[k])) * dx < X) ++m[k];
+    }
+    const int d = n - (a + m[0] + m[1]);
+    if (d >= 0) {
+      c = Counts{{m[0], m[1], a}};
+      left = d;
+      break;
+    }
+    a += d;  // too far: at least as many dominant crossings back
+  }
+  for (; left > 0; --left) {
+    const Around r = around(s, park, c);
+    if (r.next[2] <= r.next[0] && r.next[2] <= r.next[1]) ++c.k[2];
+    else if (r.next[0] <= r.next[1]) ++c.k[0];
+    else ++c.k[1];
+  }
+  return c;
+}
+
+// Crossings per chunk, for the warp's 32 rays.  The FP32 error of a position grows
+// with the chunk's share of the ray: an eighth keeps 2e-5 of the image maximum /
+// 1000 on 64-voxel volumes (a whole ray in one frame: 3.8e-5), and chunks of 121
+// crossings on 512-voxel ones (quarters of those rays, 1 to 3 % faster, do not).
+__device__ __forceinline__ int chunk_steps(const SlabRay& s) {
+  const int most = __reduce_max_sync(0xffffffffu, s.cnt[0] + s.cnt[1] + s.cnt[2]);
+  constexpr int kBlock = kChunks * kFwdUnroll;
+  return max((most + kBlock - 1) / kBlock, most > 512 ? 120 / kFwdUnroll : 1) * kFwdUnroll + 1;
+}
+
+// Chunks [q0, q1) of the ray, `size` crossings each, chunk q's sum to sink(q, sum);
+// the last chunk goes on to the exit.
+template <int DT, class Sink>
+__device__ __forceinline__ void walk_forward(const VolumeDev& vd, const SlabRay& s, const FwdPark* park, int size, int q0,
+                                             int q1, Sink sink) {
+  const int total = s.cnt[0] + s.cnt[1] + s.cnt[2];
+  if (q0 > 0 && q0 * size >= total) return;
+  Counts c = q0 > 0 ? counts_after(s, park, q0 * size) : Counts{{0, 0, 0}};
+  Around ar = around(s, park, c);
+  int off = s.off + c.k[0] * s.step[0] + c.k[1] * s.step[1] + c.k[2] * s.step[2];
+  float v = gather<DT>(vd, off);
+  int todo = total - q0 * size;  // crossings from here on
+  float ac = s.start;
+  for (int q = q0; q < q1; ++q) {
+    const u64 O = static_cast<u64>(static_cast<u32>(c.k[2])) << 32;  // the last dominant plane
+    if (q > 0) ac = fix_to_float(static_cast<long long>(ar.at - O));
+    const float x0 = fix_to_float(static_cast<long long>(ar.next[0] - O)),
+                x1 = fix_to_float(static_cast<long long>(ar.next[1] - O));
+    const int n = min(todo, size);
+    float acc = 0.f;
+    if (n > 0) {
+      float tx = 1.f, ty = x0, tz = x1, ly = 0.f, lz = 0.f;
+#define DRR_FSTEP(an)                                                                   \
+  const float an = walk_step(tx, ty, tz, ly, lz, off, s.step[2], s.step[0], s.step[1]); \
+  next_xy(ty, tz, ly, lz, s.r0, s.r1, x0, x1);
+      DRR_FSTEP(a1)
+      float an1 = a1;
+      float v1 = gather<DT>(vd, off);
+#pragma unroll kFwdUnroll
+      for (int i = 1; i < n; ++i) {
+        DRR_FSTEP(an2)
+        const float v2 = gather<DT>(vd, off);
+        acc = fmaf(an1 - ac, v, acc);
+        ac = an1;
+        an1 = an2;
+        v = v1;
+        v1 = v2;
+      }
+#undef DRR_FSTEP
+      todo -= n;
+      c.k[2] += static_cast<int>(tx) - 1;
+      c.k[0] += static_cast<int>(ly);
+      c.k[1] += static_cast<int>(lz);
+      ar = around(s, park, c);
+      if (!ar.ordered) {  // FP32 took the chunk's last crossings in another order
+        c = counts_after(s, park, total - todo);
+        ar = around(s, park, c);
+        off = s.off + c.k[0] * s.step[0] + c.k[1] * s.step[1] + c.k[2] * s.step[2];
+        v1 = gather<DT>(vd, off);
+      }
+      const float at = fix_to_float(static_cast<long long>(ar.at - O));
+      acc = fmaf(at - ac, v, acc);  // the segment that ends at the chunk's last crossing, exact end
+      ac = at;
+      v = v1;
+    }
+    if (todo == 0) {  // the segment up to the exit
+      sink(q, fmaf(fix_to_float(static_cast<long long>(s.qx - O)) - ac, v, acc));
+      return;
+    }
+    sink(q, acc);
+  }
 }
 
 // The loops are cut into np pieces: piece p takes of each slot the planes
@@ -1232,12 +1348,19 @@ struct ExactRay {
 
 // Crossings of an axis (first one at A, spacing D, cnt of them) that precede
 // position pos: those at a smaller position, and with `tie` those at the same one.
-__device__ __forceinline__ int count_before(u64 pos, bool tie, u64 A, u64 D, int cnt, float rd) {
-  if (cnt <= 0 || pos < A) return 0;
-  int n = min(static_cast<int>(fix_to_float(static_cast<long long>(pos - A)) * rd), cnt);
-  while (n < cnt && (fix_at(A, D, static_cast<u32>(n)) < pos || (tie && fix_at(A, D, static_cast<u32>(n)) == pos))) ++n;
-  while (n > 0 && !(fix_at(A, D, static_cast<u32>(n - 1)) < pos || (tie && fix_at(A, D, static_cast<u32>(n - 1)) == pos))) --n;
-  return n;
+// The FP32 quotient is off by less than one (cnt below 2^20; checked by the caller
+// through `loop`), so three candidates decide, without a branch.
+__device__ __forceinline__ int count_before(u64 pos, bool tie, u64 A, u64 D, int cnt, float rd, bool loop) {
+  const u64 lim = pos + (tie ? 1ull : 0ull);  // crossings below it count
+  const int est = lim > A ? static_cast<int>(fix_to_float(static_cast<long long>(lim - A)) * rd) : 0;
+  int n = max(min(est, cnt) - 1, 0);
+  if (loop) {
+    while (n < cnt && fix_at(A, D, static_cast<u32>(n)) < lim) ++n;
+    while (n > 0 && fix_at(A, D, static_cast<u32>(n - 1)) >= lim) --n;
+    return n;
+  }
+  const u64 x = fix_at(A, D, static_cast<u32>(n));
+  return n + (n < cnt && x < lim) + (n + 1 < cnt && x + D < lim) + (n + 2 < cnt && x + 2ull * D < lim);
 }
 
 // The rays of `mask` (lanes of the warp, each lane's pixel in h, w) in exact
@@ -1269,6 +1392,7 @@ __device__ __noinline__ void exact_rays(const VolumeDev& vd, const PoseGeom& pg,
       x.c = static_cast<float>(1.0 - 2.0 * r.amin);
       if (r.cnt[1] > r.cnt[0]) q.dom = 1;
       if (r.cnt[2] > max(r.cnt[0], r.cnt[1])) q.dom = 2;
+      const bool many = max(max(r.cnt[0], r.cnt[1]), r.cnt[2]) >= (1 << 20);
       float rd[3];
       u64 first = kFixMax;
 #pragma unroll
@@ -1284,10 +1408,11 @@ __device__ __noinline__ void exact_rays(const VolumeDev& vd, const PoseGeom& pg,
       for (int a = 0; a < 3; ++a) {
         const int b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;
         float G = 0.f, A = 0.f;
+#pragma unroll 4
         for (int k = lane; k < r.cnt[a]; k += 32) {
           const u64 pos = fix_at(r.A0[a], r.D[a], static_cast<u32>(k));
-          const int nb = count_before(pos, b < a, r.A0[b], r.D[b], r.cnt[b], rd[b]);
-          const int nc = count_before(pos, c < a, r.A0[c], r.D[c], r.cnt[c], rd[c]);
+          const int nb = count_before(pos, b < a, r.A0[b], r.D[b], r.cnt[b], rd[b], many);
+          const int nc = count_before(pos, c < a, r.A0[c], r.D[c], r.cnt[c], rd[c], many);
           const int off = r.off + k * r.step[a] + nb * r.step[b] + nc * r.step[c];
           const float vb = gather<DT>(vd, off), va = gather<DT>(vd, off + r.step[a]);
           u64 next = kFixMax;  // the end of the segment after the crossing
@@ -1628,6 +1753,22 @@ __device__ __forceinline__ bool walk_pieces(const VolumeDev& vd, const SlabRay& 
   return near;
 }
 
+// The DRR value from the sum of a ray's chunks (all 32 lanes call; rs as
+// slab_setup returned it).
+template <int DT>
+__device__ __forceinline__ float forward_finish(const VolumeDev& vd, const PoseGeom& pg, int h, int w, int rs,
+                                                const SlabRay& s, float F) {
+  const bool exact = rs > 0 && (s.exact || !(fabsf(F) <= 3.0e38f));  // a voxel that is not finite: segment by segment
+  const u32 mask = __ballot_sync(0xffffffffu, exact);
+  F *= s.rg2;
+  if (mask) {
+    ExactRay x;
+    exact_rays<DT>(vd, pg, mask, h, w, &x);
+    if (exact) F = x.q.F;
+  }
+  return rs < 0 ? __int_as_float(0x7fffffff) : (rs > 0 ? F * s.len * vd.out_scale : 0.f);
+}
+
 // The rays of one warp tile (all 32 lanes call; a lane outside the detector
 // passes valid = false).
 template <int MODE, int DT>
@@ -1637,14 +1778,13 @@ __device__ __forceinline__ void trace_tile(const VolumeDev& vd, const PoseGeom& 
 #pragma unroll
   for (int k = 0; k < 6; ++k) res.J[k] = 0.f;
   if constexpr (MODE == kFwd) {
-    RaySetup r;
-    const int rs = valid ? ray_setup(vd, pg, h, w, r) : 0;
-    if (rs < 0) {
-      res.F = __int_as_float(0x7fffffff);
-    } else if (rs > 0) {
-      const float L = sqrtf(fmaf(r.d[2], r.d[2], fmaf(r.d[1], r.d[1], r.d[0] * r.d[0])));
-      res.F = walk_forward<DT>(vd, r, park) * L * vd.out_scale;
-    }
+    SlabRay s;
+    const int rs = valid ? slab_setup<kFwd>(vd, pg, gf, h, w, s, park) : 0;
+    if (rs <= 0) slab_idle(vd, s);
+    const int size = chunk_steps(s);
+    float F = 0.f;
+    if (rs > 0) walk_forward<DT>(vd, s, park, size, 0, kChunks, [&](int, float acc) { F += acc; });
+    res.F = forward_finish<DT>(vd, pg, h, w, rs, s, F);
   } else {
     SlabRay s;
     const int rs = valid ? slab_setup<MODE>(vd, pg, gf, h, w, s, park) : 0;
@@ -1679,7 +1819,7 @@ __global__ void __launch_bounds__(kThreads, (MODE == kFwdJac || MODE == kPoseGra
                   float* __restrict__ partials, float* __restrict__ gvol) {
   __shared__ PoseGeom spg[kThreads / 32];
   constexpr bool kBp = MODE == kBackproject;
-  constexpr bool kSlab = std::is_same_v<typename ParkFor<MODE>::type, Park>;
+  constexpr bool kSlab = !std::is_same_v<typename ParkFor<MODE>::type, WalkScratch>;
   __shared__ typename ParkFor<MODE>::type ws;
   __shared__ GeomFF sgf[kSlab ? kThreads / 32 : 1];
   grid_dep_wait();
@@ -1751,24 +1891,25 @@ __global__ void __launch_bounds__(kThreads, (MODE == kFwdJac || MODE == kPoseGra
 }
 
 // ---------------------------------------------------------------------------
-// Split walk for launches too small to fill the GPU (the fused forward +
-// pose-Jacobian mode): a block of K warps takes
+// Split walk for launches too small to fill the GPU (modes kFwd and kFwdJac): a
+// block of K warps takes
 // one warp tile (8x4 pixels, pose-major); every warp sets up the tile's 32 rays
 // and sums its share of the loops' pieces, which it parks in shared memory, and
 // the first warp adds each ray's pieces in piece order and finishes the rays.
 // The sums and their order are trace_tile's, so the results are the same bits.
 // ---------------------------------------------------------------------------
-template <int DT, int K>
+template <int MODE, int DT, int K>
 __global__ void __launch_bounds__(32 * K) siddon_split_kernel(VolumeDev vd, DetDev det, const PoseGeom* __restrict__ pgs,
                                                               int B, unsigned int* __restrict__ counter,
                                                               float* __restrict__ out, float* __restrict__ jac) {
   __shared__ PoseGeom pg;
   __shared__ GeomFF gf;
-  __shared__ Park park;  // indexed by threadIdx.x (< 32 K)
-  __shared__ struct {
-    float3 minor[2][32];
+  __shared__ typename ParkFor<MODE>::type park;  // indexed by threadIdx.x (< 32 K)
+  struct Piece {
     float S[32];
-  } piece[kPieces];
+    float3 minor[MODE == kFwd ? 1 : 2][32];
+  };
+  __shared__ Piece piece[MODE == kFwd ? kChunks : kPieces];
   __shared__ unsigned int exact_s[K];
   __shared__ unsigned int tile_s;
   grid_dep_wait();
@@ -1799,42 +1940,58 @@ __global__ void __launch_bounds__(32 * K) siddon_split_kernel(VolumeDev vd, DetD
     const int h = ty * kWarpTileH + lane / kWarpTileW, w = tx * kWarpTileW + lane % kWarpTileW;
     const bool valid = (w < det.W) && (h < det.H);
     SlabRay s;
-    const int rs = valid ? slab_setup<kFwdJac>(vd, pg, gf, h, w, s, &park) : 0;
+    const int rs = valid ? slab_setup<MODE>(vd, pg, gf, h, w, s, &park) : 0;
     if (rs <= 0) slab_idle(vd, s);
-    bool exact = s.exact;
-    const Plan pl = plan_pieces(s);
-    // this warp's share of the pieces
-    exact |= walk_pieces<DT>(vd, s, pl, pl.np * warp / K, pl.np * (warp + 1) / K,
-                                   [&](int p, int slot, const MinorSums& r) {
-                                     if (slot == 2) piece[p].S[lane] = r.g;
-                                     else piece[p].minor[slot][lane] = make_float3(r.g, r.c, r.h);
-                                   });
-    const unsigned int ex = __ballot_sync(0xffffffffu, exact);
-    if (lane == 0) exact_s[warp] = ex;
-    __syncthreads();
-    if (warp == 0) {
-      RayResult r;
-      r.F = rs < 0 ? __int_as_float(0x7fffffff) : 0.f;
-#pragma unroll
-      for (int k = 0; k < 6; ++k) r.J[k] = r.F;
-      SlabTotals T{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      for (int p = 0; p < pl.np; ++p) {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const float3 q = piece[p].minor[k][lane];
-          T.add(k, MinorSums{q.x, q.y, q.z, 0u});
-        }
-        T.add(2, MinorSums{piece[p].S[lane], 0.f, 0.f, 0u});
+    RayResult r;
+    if constexpr (MODE == kFwd) {
+      const int size = chunk_steps(s), total = s.cnt[0] + s.cnt[1] + s.cnt[2];
+      if (rs > 0)
+        walk_forward<DT>(vd, s, &park, size, (kChunks * warp + K - 1) / K, (kChunks * (warp + 1) + K - 1) / K,
+                         [&](int q, float acc) { piece[q].S[lane] = acc; });
+      __syncthreads();
+      if (warp == 0) {
+        float F = 0.f;
+        if (rs > 0)
+          for (int q = 0; q == 0 || q * size < total; ++q) F += piece[q].S[lane];
+        r.F = forward_finish<DT>(vd, pg, h, w, rs, s, F);
       }
-      unsigned int any = 0u;
+    } else {
+      bool exact = s.exact;
+      const Plan pl = plan_pieces(s);
+      // this warp's share of the pieces
+      exact |= walk_pieces<DT>(vd, s, pl, pl.np * warp / K, pl.np * (warp + 1) / K,
+                                     [&](int p, int slot, const MinorSums& r) {
+                                       if (slot == 2) piece[p].S[lane] = r.g;
+                                       else piece[p].minor[slot][lane] = make_float3(r.g, r.c, r.h);
+                                     });
+      const unsigned int ex = __ballot_sync(0xffffffffu, exact);
+      if (lane == 0) exact_s[warp] = ex;
+      __syncthreads();
+      if (warp == 0) {
+        r.F = rs < 0 ? __int_as_float(0x7fffffff) : 0.f;
 #pragma unroll
-      for (int k = 0; k < K; ++k) any |= exact_s[k];
-      JacSums q;
-      slab_finish<kFwdJac, DT>(vd, pg, h, w, rs > 0, s, T, (any >> lane) & 1u, &park, q);
-      if (rs > 0) ray_outputs<kFwdJac>(vd, pg, h, w, q, &park, r);
-      if (valid) {
-        const size_t pix = static_cast<size_t>(h) * det.W + w;
-        out[b * npix + pix] = r.F;
+        for (int k = 0; k < 6; ++k) r.J[k] = r.F;
+        SlabTotals T{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        for (int p = 0; p < pl.np; ++p) {
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const float3 q = piece[p].minor[k][lane];
+            T.add(k, MinorSums{q.x, q.y, q.z, 0u});
+          }
+          T.add(2, MinorSums{piece[p].S[lane], 0.f, 0.f, 0u});
+        }
+        unsigned int any = 0u;
+#pragma unroll
+        for (int k = 0; k < K; ++k) any |= exact_s[k];
+        JacSums q;
+        slab_finish<kFwdJac, DT>(vd, pg, h, w, rs > 0, s, T, (any >> lane) & 1u, &park, q);
+        if (rs > 0) ray_outputs<kFwdJac>(vd, pg, h, w, q, &park, r);
+      }
+    }
+    if (warp == 0 && valid) {
+      const size_t pix = static_cast<size_t>(h) * det.W + w;
+      out[b * npix + pix] = r.F;
+      if (MODE == kFwdJac) {
 #pragma unroll
         for (int k = 0; k < 6; ++k) jac[(static_cast<size_t>(b) * 6 + k) * npix + pix] = r.J[k];
       }
@@ -2230,7 +2387,7 @@ int resident_blocks() {
 
 // The split kernel with K warps per tile: the blocks of it the device holds at
 // once (cached per device).
-template <int DT, int K>
+template <int MODE, int DT, int K>
 int split_resident_blocks() {
   constexpr int kMaxDev = 64;
   static std::atomic<int> cache[kMaxDev] = {};  // calls from several host threads may race to fill it
@@ -2240,7 +2397,7 @@ int split_resident_blocks() {
   if (v == 0) {
     int sms = 0, per_sm = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, siddon_split_kernel<DT, K>, 32 * K, 0) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, siddon_split_kernel<MODE, DT, K>, 32 * K, 0) !=
         cudaSuccess) {
       cudaGetLastError();
       v = -1;
@@ -2252,24 +2409,24 @@ int split_resident_blocks() {
   return v > 0 ? v : 0;
 }
 
-template <int DT, int K>
+template <int MODE, int DT, int K>
 cudaError_t launch_split(const VolumeDev& vd, const DetDev& det, const PoseGeom* pg, int B, unsigned int* counter,
                          float* out, float* jac, cudaStream_t stream) {
   const int64_t tiles = static_cast<int64_t>(pose_tiles(det)) * B;
-  const int grid = static_cast<int>(std::min<int64_t>(tiles, split_resident_blocks<DT, K>()));
-  return launch_pdl(siddon_split_kernel<DT, K>, dim3(grid), dim3(32 * K), stream, vd, det, pg, B, counter, out,
+  const int grid = static_cast<int>(std::min<int64_t>(tiles, split_resident_blocks<MODE, DT, K>()));
+  return launch_pdl(siddon_split_kernel<MODE, DT, K>, dim3(grid), dim3(32 * K), stream, vd, det, pg, B, counter, out,
                     jac);
 }
 
-// Warps per ray (per warp tile) for a fused forward + Jacobian launch: 8 or 4 when the split
+// Warps per ray (per warp tile) for a render launch: 8 or 4 when the split
 // kernel's resident blocks can take every tile of the launch at once (the
 // whole-ray walk would leave most of the GPU idle, latency-bound on few warps),
 // 1 otherwise.
-template <int DT>
+template <int MODE, int DT>
 int split_lanes(const DetDev& det, int B) {
   const int64_t tiles = static_cast<int64_t>(pose_tiles(det)) * B;
-  if (tiles <= split_resident_blocks<DT, 8>()) return 8;
-  if (tiles <= split_resident_blocks<DT, 4>()) return 4;
+  if (tiles <= split_resident_blocks<MODE, DT, 8>()) return 8;
+  if (tiles <= split_resident_blocks<MODE, DT, 4>()) return 4;
   return 1;
 }
 
@@ -2277,9 +2434,9 @@ template <int MODE, int DT>
 cudaError_t launch_siddon_dt(const VolumeDev& vd, const DetDev& det, const PoseGeom* pg, int B, unsigned int* counter,
                              float* out, float* jac, const float* gin, float* partials, float* gvol,
                              cudaStream_t stream, int lanes = 1) {
-  if constexpr (MODE == kFwdJac) {
-    if (lanes == 8) return launch_split<DT, 8>(vd, det, pg, B, counter, out, jac, stream);
-    if (lanes == 4) return launch_split<DT, 4>(vd, det, pg, B, counter, out, jac, stream);
+  if constexpr (MODE == kFwd || MODE == kFwdJac) {
+    if (lanes == 8) return launch_split<MODE, DT, 8>(vd, det, pg, B, counter, out, jac, stream);
+    if (lanes == 4) return launch_split<MODE, DT, 4>(vd, det, pg, B, counter, out, jac, stream);
   }
   const int64_t tiles = static_cast<int64_t>(pose_tiles(det)) * B;
   const int64_t want = (tiles + kThreads / 32 - 1) / (kThreads / 32);
@@ -2445,18 +2602,25 @@ cudaError_t launch_ray_setup(const float* poses, int B, const DetDev& det, float
   return cudaGetLastError();
 }
 
-int render_split_lanes(const VolumeDev& vd, const DetDev& det, int B) {
+namespace {
+template <int MODE>
+int mode_split_lanes(const VolumeDev& vd, const DetDev& det, int B) {
   switch (vd.dtype) {
-    case kF32: return split_lanes<kF32>(det, B);
-    case kBF16: return split_lanes<kBF16>(det, B);
-    default: return split_lanes<kF16>(det, B);
+    case kF32: return split_lanes<MODE, kF32>(det, B);
+    case kBF16: return split_lanes<MODE, kBF16>(det, B);
+    default: return split_lanes<MODE, kF16>(det, B);
   }
+}
+}  // namespace
+
+int render_split_lanes(const VolumeDev& vd, const DetDev& det, int B, bool jacobian) {
+  return jacobian ? mode_split_lanes<kFwdJac>(vd, det, B) : mode_split_lanes<kFwd>(vd, det, B);
 }
 
 cudaError_t launch_render(const VolumeDev& vd, const DetDev& det, const PoseGeom* pg, int B, float* out, float* jac,
                           cudaStream_t stream, int lanes) {
   if (jac) return launch_siddon<kFwdJac>(vd, det, pg, B, out, jac, nullptr, nullptr, nullptr, stream, lanes);
-  return launch_siddon<kFwd>(vd, det, pg, B, out, nullptr, nullptr, nullptr, nullptr, stream);
+  return launch_siddon<kFwd>(vd, det, pg, B, out, nullptr, nullptr, nullptr, nullptr, stream, lanes);
 }
 
 cudaError_t launch_pose_grad_walk(const VolumeDev& vd, const DetDev& det, const PoseGeom* pg, int B,

@@ -280,7 +280,7 @@ cudaError_t drr_server_s::launch_registration_step(const Req& q, cudaStream_t ks
   const int B = q.r.B;
   cudaError_t e = drr::launch_pose_setup(q.d_poses, B, q.det, &vd, q.d_geom, ks);
   if (e == cudaSuccess)
-    e = drr::launch_render(vd, q.det, q.d_geom, B, q.d_e, q.d_jac, ks, drr::render_split_lanes(vd, q.det, B));
+    e = drr::launch_render(vd, q.det, q.d_geom, B, q.d_e, q.d_jac, ks, drr::render_split_lanes(vd, q.det, B, true));
   if (e == cudaSuccess)
     e = drr::launch_zncc(q.d_e, q.d_fixed, q.npix, B, static_cast<int>(q.npix), q.r.zncc_eps, q.d_loss, q.d_grad, ks);
   if (e == cudaSuccess) e = drr::launch_pose_grad_from_jacobian(q.det, B, q.d_grad, q.d_jac, q.d_gpose, ks);

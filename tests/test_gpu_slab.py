@@ -1,5 +1,5 @@
 """The slab walk of the Jacobian modes (each axis' crossings in a loop of its own)
-where it can go wrong: volumes of one to three voxels along an axis, strong
+and the forward walk where they can go wrong: volumes of one to three voxels along an axis, strong
 anisotropy (an axis crossed once or never), rays parallel or almost parallel to
 voxel planes, crossings that coincide on a lattice, a source inside the volume,
 ragged detectors, and voxels that are not finite.  Against the FP64 oracle, with
@@ -88,3 +88,37 @@ def test_voxels_that_are_not_finite_reach_only_their_rays(drr, bad):
     np.testing.assert_array_equal(np.isfinite(E), np.isfinite(F))
     np.testing.assert_array_equal(E[~np.isfinite(F)], F[~np.isfinite(F)])
     np.testing.assert_allclose(E[np.isfinite(F)], F[np.isfinite(F)], rtol=FP32_TOL, atol=1e-3 * FP32_TOL)
+
+
+@pytest.mark.parametrize("layout", ["x", "y"])
+@pytest.mark.parametrize("name", list(CASES))
+def test_forward_walk_against_the_oracle(drr, name, layout):
+    # a small launch (split over the warps of a tile) and one that fills the GPU give the
+    # same bits, with ties at the ends of chunks among them, and both match the oracle
+    shape, sp, det, poses_np, _ = CASES[name]
+    vol_np = _noise(shape, len(name))
+    vol = drr.Volume(vol_np, sp, layout=layout)
+    B = poses_np.shape[0]
+    E = drr.render(vol, det, torch.from_numpy(poses_np).cuda()).cpu().numpy()
+    assert rel_err(E, oracle.render(ovol(vol_np, sp), odet(det), poses_np)).max() < FP32_TOL
+    tiles = -(-det.height // 4) * -(-det.width // 8) * B
+    many = -(-6000 // tiles)  # past the split kernel's resident tiles
+    F = drr.render(vol, det, torch.from_numpy(np.tile(poses_np, (many, 1))).cuda()).cpu().numpy()
+    np.testing.assert_array_equal(F.reshape(many, *E.shape), np.broadcast_to(E, (many, *E.shape)))
+
+
+def test_forward_walk_of_long_rays(drr):
+    # more crossings than one FP32 frame would hold: 1500 planes along the rays
+    vol_np = _noise((3, 40, 1500), 5)
+    vol = drr.Volume(vol_np, (0.2, 0.25, 1.0))
+    det = inputs.Detector(700.0, 9, 17, 0.4, 0.4)
+    poses_np = np.array([[0.01, 0.002, 0.1, 0.0, 0.3, 0.1], [0.004, -0.001, 0.0, 1.0, 0.0, 0.0]], np.float32)
+    P = torch.from_numpy(poses_np).cuda()
+    ov = ovol(vol_np, (0.2, 0.25, 1.0))
+    E_ref, J_ref = oracle.render(ov, odet(det), poses_np, jacobian=True)
+    assert rel_err(drr.render(vol, det, P).cpu().numpy(), E_ref).max() < FP32_TOL
+    E, J = drr.render(vol, det, P, jacobian=True)
+    assert rel_err(E.cpu().numpy(), E_ref).max() < FP32_TOL
+    J_ref = np.moveaxis(J_ref, -1, 1)
+    for grp in (slice(0, 3), slice(3, 6)):
+        assert (np.abs(J.cpu().numpy()[:, grp] - J_ref[:, grp]) / np.abs(J_ref[:, grp]).max()).max() < GRAD_TOL
