@@ -165,42 +165,34 @@ __device__ void apply3f(const float* A, const float* x, float* y) {
   for (int r = 0; r < 3; ++r) y[r] = fmaf(A[3 * r], x[0], fmaf(A[3 * r + 1], x[1], A[3 * r + 2] * x[2]));
 }
 
-// FP32 chain-rule terms of one pose (dR/d eta_j applied to s_c, p_c - s_c and the
-// pixel steps), from the FP32-rounded sines and cosines: they are stored as FP32.
-__device__ void chain_terms(const float cs[6], const float t[3], double rho, double pw, double ph, const DetDev& det,
-                            PoseGeom* g) {
+// FP32 chain-rule terms of one angle j of a pose (dR/d eta_j applied to s_c, p_c -
+// s_c and the pixel steps), from the FP32-rounded sines and cosines: they are
+// stored as FP32.  One lane per angle: dR_j is the product of the three rotations
+// with the j-th replaced by its derivative.
+__device__ void chain_terms(int j, const float cs[6], double rho, double pw, double ph, const DetDev& det, PoseGeom* g) {
   const float sz = cs[0], cz = cs[1], sy = cs[2], cy = cs[3], sx = cs[4], cx = cs[5];
-  const float Rz[9] = {cz, -sz, 0.f, sz, cz, 0.f, 0.f, 0.f, 1.f};
-  const float Ry[9] = {cy, 0.f, sy, 0.f, 1.f, 0.f, -sy, 0.f, cy};
-  const float Rx[9] = {1.f, 0.f, 0.f, 0.f, cx, -sx, 0.f, sx, cx};
-  const float dRz[9] = {-sz, -cz, 0.f, cz, -sz, 0.f, 0.f, 0.f, 0.f};
-  const float dRy[9] = {-sy, 0.f, cy, 0.f, 0.f, 0.f, -cy, 0.f, -sy};
-  const float dRx[9] = {0.f, 0.f, 0.f, 0.f, -sx, -cx, 0.f, cx, -sx};
-  float T[9], U[9], dR[27];
-  mul3f(Rz, Ry, T);
-  mul3f(dRz, Ry, U);
-  mul3f(U, Rx, dR);
-  mul3f(Rz, dRy, U);
-  mul3f(U, Rx, dR + 9);
-  mul3f(T, dRx, dR + 18);
-  // angular velocities of the three angles in the world frame, dR_j R^T x =
-  // omega_j x x: rz turns about e_z, ry about Rz e_y, rx about Rz Ry e_x
-  const float om[9] = {0.f, 0.f, 1.f, -sz, cz, 0.f, cz * cy, sz * cy, -sy};
+  const bool d0 = j == 0, d1 = j == 1, d2 = j == 2;
+  // [c -s; s c] or its derivative [-s -c; c -s], embedded in the rotation's plane
+  const float zc = d0 ? -sz : cz, zs = d0 ? cz : sz, z1 = d0 ? 0.f : 1.f;
+  const float yc = d1 ? -sy : cy, ys = d1 ? cy : sy, y1 = d1 ? 0.f : 1.f;
+  const float xc = d2 ? -sx : cx, xs = d2 ? cx : sx, x1 = d2 ? 0.f : 1.f;
+  const float Z[9] = {zc, -zs, 0.f, zs, zc, 0.f, 0.f, 0.f, z1};
+  const float Y[9] = {yc, 0.f, ys, 0.f, y1, 0.f, -ys, 0.f, yc};
+  const float X[9] = {x1, 0.f, 0.f, 0.f, xc, -xs, 0.f, xs, xc};
+  float T[9], dR[9];
+  mul3f(Z, Y, T);
+  mul3f(T, X, dR);
+  // angular velocity of the angle in the world frame, dR_j R^T x = omega_j x x:
+  // rz turns about e_z, ry about Rz e_y, rx about Rz Ry e_x
+  g->Om[j][0] = d0 ? 0.f : (d1 ? -sz : cz * cy);
+  g->Om[j][1] = d0 ? 0.f : (d1 ? cz : sz * cy);
+  g->Om[j][2] = d0 ? 1.f : (d1 ? 0.f : -sy);
   const float q[3] = {static_cast<float>(-2.0 * rho), static_cast<float>(pw), static_cast<float>(ph)};
   const float vw[3] = {0.f, det.dw, 0.f};
   const float vh[3] = {0.f, 0.f, det.dh};
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) g->Om[j][a] = om[3 * j + a];
-    apply3f(dR + 9 * j, q, g->Q[j]);
-    apply3f(dR + 9 * j, vw, g->Wv[j]);
-    apply3f(dR + 9 * j, vh, g->Hv[j]);
-  }
-#pragma unroll
-  for (int a = 0; a < 3; ++a) g->t[a] = t[a];
-  g->hc = 0.5f * static_cast<float>(det.H - 1);
-  g->wc = 0.5f * static_cast<float>(det.W - 1);
+  apply3f(dR, q, g->Q[j]);
+  apply3f(dR, vw, g->Wv[j]);
+  apply3f(dR, vh, g->Hv[j]);
 }
 
 // Per-pose geometry in the volume's voxel units plus the chain-rule terms,
@@ -231,28 +223,32 @@ __device__ void warp_pose_geom(const float* pose, const DetDev& det, const Volum
     const double p00 = fma(ph, r2, fma(pw, r1, fma(-rho, r0, t)));     // R pc00 + t
     const double ew = static_cast<double>(det.dw) * r1;                 // R (0, dw, 0)
     const double eh = static_cast<double>(det.dh) * r2;                 // R (0, 0, dh)
-    const double dl = static_cast<double>(pick3(a, vd.delta[0], vd.delta[1], vd.delta[2]));
+    const double dl = static_cast<double>(pick3(a, vd.delta[0], vd.delta[1], vd.delta[2])), rd = 1.0 / dl;
     const int na = pick3(a, vd.n[0], vd.n[1], vd.n[2]);
     const double lo = -0.5 * static_cast<double>(na) * dl;  // b_a: volume centred at the origin
-    const double u0 = (s - lo) / dl;
+    const double u0 = (s - lo) * rd;
     const double un = static_cast<double>(na) - u0;
     g->u0[a] = u0;
     g->un[a] = un;
     g->u0f[a] = static_cast<float>(u0);
     g->unf[a] = static_cast<float>(un);
-    g->g00[a] = (p00 - s) / dl;
-    g->gw[a] = ew / dl;
-    g->gh[a] = eh / dl;
+    g->g00[a] = (p00 - s) * rd;
+    g->gw[a] = ew * rd;
+    g->gh[a] = eh * rd;
   }
   // columns of R (R e_x, R e_y, R e_z) for the detector-parameter chain
 #pragma unroll
   for (int i = 0; i < 9; ++i)
     if (lane == i) g->Rc[i % 3][i / 3] = static_cast<float>(R[i]);
-  if (lane == 0) {
+  if (lane < 3) {
     const float cs[6] = {static_cast<float>(sz), static_cast<float>(cz), static_cast<float>(sy),
                          static_cast<float>(cy), static_cast<float>(sx), static_cast<float>(cx)};
-    const float tr[3] = {pose[3], pose[4], pose[5]};
-    chain_terms(cs, tr, rho, pw, ph, det, g);
+    g->t[lane] = pose[3 + lane];
+    chain_terms(lane, cs, rho, pw, ph, det, g);
+  }
+  if (lane == 3) {
+    g->hc = 0.5f * static_cast<float>(det.H - 1);
+    g->wc = 0.5f * static_cast<float>(det.W - 1);
   }
 }
 
@@ -2095,34 +2091,47 @@ __global__ void __cluster_dims__(kJacCluster, 1, 1) __launch_bounds__(kJacThread
   }
 }
 
-// Fixed-order FP64 sum of one pose's per-tile partial sums (nt tiles, ncol
-// values each, tile-major): thread t adds tiles t, t + kFinThreads, ... in
-// order (one coalesced pass for all columns), each warp's sums are combined by
-// a fixed shuffle tree, and thread k adds the warps' sums of column k in warp
-// order.  The order depends only on nt, so the result is bitwise reproducible,
-// and the server and the direct calls, which both finish through here, agree
-// bit for bit.  Called by all threads of the block.
+// Fixed-order sum of one pose's per-tile partial sums (nt tiles, ncol values each,
+// tile-major) to FP64 accuracy: thread t adds tiles t, t + kFinThreads, ... in
+// order (one coalesced pass for all columns), each warp's sums are combined by a
+// fixed shuffle tree, and thread k adds the warps' sums of column k in warp order.
+// The order depends only on nt, so the result is bitwise reproducible, and the
+// server and the direct calls, which both finish through here, agree bit for
+// bit.  Called by all threads of the block.  The sums run as value + error pairs
+// of FP32 (exact but for the rounding of the error, ~2^-46 of the sum) up to the
+// warps' totals: as FP64 additions they bounded the kernel (15 us for 3 poses of
+// 2720 tiles; this GPU issues FP64 at 1/64 of the FP32 rate).
 constexpr int kFinThreads = 256;
 
 __device__ __forceinline__ void sum_pose_partials(const float* __restrict__ p, int nt, int ncol,
                                                   float* __restrict__ out) {
   __shared__ double wsum[kFinThreads / 32][6];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  double s[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  float2 s[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) s[k] = make_float2(0.f, 0.f);
+#pragma unroll 4
   for (int c = t; c < nt; c += kFinThreads) {
     const float* row = p + static_cast<size_t>(c) * ncol;
 #pragma unroll
-    for (int k = 0; k < 6; ++k)
-      if (k < ncol) s[k] += static_cast<double>(row[k]);
+    for (int k = 0; k < 6; ++k) {
+      if (k < ncol) {
+        const float2 x = ff_sum(s[k].x, row[k]);
+        s[k] = make_float2(x.x, __fadd_rn(s[k].y, x.y));
+      }
+    }
   }
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+    for (int o = 16; o > 0; o >>= 1) {
+      const float2 x = ff_sum(s[k].x, __shfl_xor_sync(0xffffffffu, s[k].x, o));
+      s[k] = make_float2(x.x, __fadd_rn(__fadd_rn(s[k].y, __shfl_xor_sync(0xffffffffu, s[k].y, o)), x.y));
+    }
   }
   if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) wsum[warp][k] = s[k];
+    for (int k = 0; k < 6; ++k) wsum[warp][k] = static_cast<double>(s[k].x) + static_cast<double>(s[k].y);
   }
   __syncthreads();
   if (t < ncol) {
@@ -2239,7 +2248,7 @@ __device__ __forceinline__ void serve_trace(const VolumeDev& vd, const PoseGeom&
 // walk, gradient tiles the Jacobian walk with the warp's sum of g . J written
 // per tile; a warp copies its request's record and pose geometry to its own
 // shared slots when they change.
-__global__ void __launch_bounds__(kThreads, 4) serve_walk_kernel(const ServeHeader* __restrict__ hdr,
+__global__ void __launch_bounds__(kThreads, 3) serve_walk_kernel(const ServeHeader* __restrict__ hdr,
                                                                  const ServeRequest* __restrict__ reqs,
                                                                  unsigned int* __restrict__ status,
                                                                  int* __restrict__ counter) {
