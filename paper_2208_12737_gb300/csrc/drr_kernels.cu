@@ -488,17 +488,13 @@ __device__ __forceinline__ int ray_setup(const VolumeDev& vd, const PoseGeom& pg
 #ifndef DRR_FWD_MINB
 #define DRR_FWD_MINB 4
 #endif
+#ifndef DRR_BP_MINB
+#define DRR_BP_MINB 4
+#endif
 #ifndef DRR_JAC_MINB
 #define DRR_JAC_MINB 3
 #endif
 constexpr float kTwoM32 = 2.3283064365386963e-10f;  // 2^-32
-
-// Per-thread exact crossing parameters of the back-projection, kept in shared
-// memory: they are read only when a chunk starts.
-struct WalkScratch {
-  unsigned long long A0[3][kThreads];
-  unsigned long long D[3][kThreads];
-};
 
 __device__ __forceinline__ unsigned long long fix_at(unsigned long long A0, unsigned long long D, unsigned int k) {
   return A0 + static_cast<unsigned long long>(k) * D;
@@ -613,10 +609,11 @@ struct FwdPark {
   u64 x0[2][kThreads], dx[2][kThreads];  // slots 0, 1: q_2 at crossing 0 and its step (32.32)
   u64 y0[2][kThreads], dy[2][kThreads];  // q_0, q_1 at dominant crossing 0 and their steps (24.40)
 };
+struct NoPark {};
 template <int MODE>
 struct ParkFor {
   using type = std::conditional_t<MODE == kFwdJac || MODE == kPoseGrad || MODE == kGeoGrad, Park,
-                                  std::conditional_t<MODE == kFwd, FwdPark, WalkScratch>>;
+                                  std::conditional_t<MODE == kFwd || MODE == kBackproject, FwdPark, NoPark>>;
 };
 
 struct SlabRay {
@@ -1628,91 +1625,173 @@ __device__ __forceinline__ void red_column_merged(float* __restrict__ gvol, unsi
   if (head && addr < nvox) atomicAdd(gvol + addr, s);
 }
 
+// Segments of the rays of `mask` in exact crossing order, as exact_rays finds them
+// (all 32 lanes share one ray's crossings; the segment after each crossing is
+// added), for the rays that slab_setup leaves to FP64.
+__device__ __noinline__ void backproject_exact(const VolumeDev& vd, const PoseGeom& pg, u32 mask, int h, int w, float g,
+                                               float* __restrict__ gvol) {
+  constexpr u32 kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const u32 nvox = static_cast<u32>(vd.n[0] * vd.n[1] * vd.n[2]);
+  for (; mask; mask &= mask - 1u) {
+    const int L = __ffs(static_cast<int>(mask)) - 1;
+    const int hh = __shfl_sync(kAll, h, L), ww = __shfl_sync(kAll, w, L);
+    const float gg = __shfl_sync(kAll, g, L);
+    RaySetup r;
+    if (ray_setup(vd, pg, hh, ww, r) <= 0) continue;  // the same for all lanes
+    const float s = gg * sqrtf(fmaf(r.d[2], r.d[2], fmaf(r.d[1], r.d[1], r.d[0] * r.d[0]))) * r.unit;
+    const bool many = max(max(r.cnt[0], r.cnt[1]), r.cnt[2]) >= (1 << 20);
+    const auto add = [&](int ix, int iy, int iz, u64 len) {
+      const u32 lin = static_cast<u32>(ix + vd.n[0] * (iy + vd.n[1] * iz));
+#if DRR_CHECK_BOUNDS
+      if (lin >= nvox) atomicOr(&g_fault_word, kFaultBackproject);
+#endif
+      if (lin < nvox) atomicAdd(gvol + lin, s * fix_to_float(static_cast<long long>(len)));
+    };
+    float rd[3];
+    int sg[3];
+    u64 first = kFixMax;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      rd[a] = 1.f / fix_to_float(static_cast<long long>(r.D[a]));
+      sg[a] = r.step[a] > 0 ? 1 : -1;
+      if (r.cnt[a] > 0) first = min(first, r.A0[a]);
+    }
+    if (lane == 0) add(r.ient[0], r.ient[1], r.ient[2], first);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;
+      for (int k = lane; k < r.cnt[a]; k += 32) {
+        const u64 pos = fix_at(r.A0[a], r.D[a], static_cast<u32>(k));
+        const int nb = count_before(pos, b < a, r.A0[b], r.D[b], r.cnt[b], rd[b], many);
+        const int nc = count_before(pos, c < a, r.A0[c], r.D[c], r.cnt[c], rd[c], many);
+        u64 next = kFixMax;  // the end of the segment after the crossing
+        if (k + 1 < r.cnt[a]) next = min(next, pos + r.D[a]);
+        if (nb < r.cnt[b]) next = min(next, fix_at(r.A0[b], r.D[b], static_cast<u32>(nb)));
+        if (nc < r.cnt[c]) next = min(next, fix_at(r.A0[c], r.D[c], static_cast<u32>(nc)));
+        int i[3];
+        i[a] = r.ient[a] + (k + 1) * sg[a];
+        i[b] = r.ient[b] + nb * sg[b];
+        i[c] = r.ient[c] + nc * sg[c];
+        add(i[0], i[1], i[2], next - pos);
+      }
+    }
+  }
+}
+
 // Back-projection walk: grad_V[voxel] += g L (a_{m+1} - a_m), the transpose of
 // the forward map V -> E (Eq. 2 is linear in V), into an unpadded (nz, ny, nx)
-// FP32 volume.  The crossings are those of the forward walk: FP32 positions
-// local to an exact fixed-point anchor, re-anchored every kBpChunk steps.  All
-// 32 lanes step together (to the warp's longest ray) and re-anchor at the same
-// steps, since their adds are merged across lanes; a lane whose pixel has no
-// ray to walk passes nseg = 0 and adds nothing.
-constexpr int kBpChunk = 64;
-__device__ __forceinline__ void walk_backproject(const VolumeDev& vd, const RaySetup& r, int nseg, float gL,
-                                                 float* __restrict__ gvol, WalkScratch* ws, int lane) {
-  const int t = threadIdx.x;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    ws->A0[a][t] = r.A0[a];
-    ws->D[a][t] = r.D[a];
-  }
-  const float dx = fix_to_float(static_cast<long long>(r.D[0])), dy = fix_to_float(static_cast<long long>(r.D[1])),
-              dz = fix_to_float(static_cast<long long>(r.D[2]));
-  // unsigned index arithmetic: a lane past its exit keeps stepping (wrapping) without adding
-  const unsigned int nx = static_cast<unsigned int>(vd.n[0]), nxy = nx * static_cast<unsigned int>(vd.n[1]);
-  const unsigned int sx = r.step[0] > 0 ? 1u : 0u - 1u;
-  const unsigned int sy = r.step[1] > 0 ? nx : 0u - nx;
-  const unsigned int sz = r.step[2] > 0 ? nxy : 0u - nxy;
-  const unsigned int nvox = static_cast<unsigned int>(vd.n[0] * vd.n[1] * vd.n[2]);
-  unsigned int lin = static_cast<unsigned int>(r.ient[0] + vd.n[0] * (r.ient[1] + vd.n[1] * r.ient[2]));
-  const float s = gL * r.unit;  // gradient per high-word unit of segment length
-  const int nmax = __reduce_max_sync(0xffffffffu, nseg);
-  unsigned int kx = 0u, ky = 0u, kz = 0u;
-  unsigned long long O = 0ull;  // exact position of the last crossing taken (the anchor)
-  float ac = 0.f;               // local position where the current segment starts
-  for (int m = 0; m < nmax;) {  // warp-uniform
-    const int n = min(nmax - m, kBpChunk);
-    const float x0 = local_pos(fix_at(ws->A0[0][t], ws->D[0][t], kx), O);
-    const float y0 = local_pos(fix_at(ws->A0[1][t], ws->D[1][t], ky), O);
-    const float z0 = local_pos(fix_at(ws->A0[2][t], ws->D[2][t], kz), O);
-    const float xe = local_pos(static_cast<unsigned long long>(kExitUnits) << 32, O);
-    float tx = x0, ty = y0, tz = z0;
-    float cx = 0.f, cy = 0.f, cz = 0.f;
-#pragma unroll 4
-    for (int j = 1; j <= n; ++j) {
-      const int step = m + j;  // this step ends segment step - 1 (the exit segment at step nseg)
-      const float an = fminf(fminf(tx, ty), tz);
-      const float val = s * ((step < nseg ? an : xe) - ac);
-#if DRR_CHECK_BOUNDS
-      if (step <= nseg && lin >= nvox) atomicOr(&g_fault_word, kFaultBackproject);
+// FP32 volume.  The crossings are those of the forward walk, in chunks from exact
+// counts (walk_forward).  All 32 lanes step together, since their adds are merged
+// across lanes, and a ray starts at the step that is its entry voxel's level, the
+// sum of the voxel indexes counted along the ray: every step adds one to it, so
+// rays of the tile that pass through a voxel do so at the same step, and their
+// adds merge.  A waiting ray takes dominant crossings before its entry; lengths
+// are clipped to [entry, exit], so those before and after the ray add nothing.
+// gL: g |p - s| alpha per dominant plane; nseg = 0: a lane without a ray.
+//
+// What bounds it: the L2's tag stage, 81 % busy with the adds (each lane's add is a
+// sector operation of its own), so the merging decides.  12 poses of 181x217 on
+// 200x216x180 voxels, forward + both gradients: 960 -> 930 us with this walk against
+// one with an FP64 ray setup whose rays all started at the first step (this kernel
+// 370 us); without the waiting 955 to 980; 3 blocks per SM 950, tiles of 2 x 16
+// pixels 927, of 4 x 8 932.
+// Waiting costs steps where a tile's rays enter at far levels (pixels many voxels
+// apart, whose rays share no voxels anyway): such tiles, more than an eighth longer
+// with it, do without.
+#ifndef DRR_BP_WAIT_SHARE
+#define DRR_BP_WAIT_SHARE 8
 #endif
-      red_column_merged<kBpTileW>(gvol, step <= nseg ? lin : 0xffffffffu, val, nvox, lane);
-      ac = an;
-      const bool bx = tx == an;
-      const bool by = !bx && ty == an;
-      const bool bz = !bx && !by;
-      lin += bx ? sx : (by ? sy : sz);
-      if (bx) cx += 1.f;
-      if (by) cy += 1.f;
-      if (bz) cz += 1.f;
-      next_xy(tx, ty, cx, cy, dx, dy, x0, y0);
-      tz = fmaf(cz, dz, z0);
+constexpr int kBpWaitShare = DRR_BP_WAIT_SHARE;
+__device__ __forceinline__ void walk_backproject(const VolumeDev& vd, const SlabRay& s, const FwdPark* park, int nseg,
+                                                 float gL, float* __restrict__ gvol, int lane) {
+  constexpr u32 kAll = 0xffffffffu;
+  const int size = chunk_steps(s);
+  // unsigned index arithmetic: a lane before its entry or past its exit keeps stepping (wrapping) without adding
+  const u32 nx = static_cast<u32>(vd.n[0]), nxy = nx * static_cast<u32>(vd.n[1]);
+  const u32 nvox = static_cast<u32>(vd.n[0] * vd.n[1] * vd.n[2]);
+  u32 st[3], entry = 0u;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int ax = k == 0 ? s.ax0 : (k == 1 ? s.ax1 : s.ax2);
+    const u32 u = pick3(ax, 1u, nx, nxy);
+    const bool up = s.step[k] > 0;
+    entry += u * static_cast<u32>(up ? s.i0[k] : pick3(ax, vd.n[0], vd.n[1], vd.n[2]) - 1 - s.i0[k]);
+    st[k] = up ? u : 0u - u;
+  }
+  const int level = s.i0[0] + s.i0[1] + s.i0[2];
+  const int first = __reduce_min_sync(kAll, nseg > 0 ? level : 0x7fffffff);
+  int wait = nseg > 0 ? level - first : 0;
+  int nmax = __reduce_max_sync(kAll, wait + nseg);
+  const int longest = __reduce_max_sync(kAll, nseg);
+  if (nmax > longest + longest / kBpWaitShare) {
+    wait = 0;
+    nmax = longest;
+  }
+  const int total = nseg - 1;
+  Counts c{{0, 0, 0}};
+  float ac = s.start;
+  u32 lin = entry;
+  for (int m = 0; m < nmax;) {  // warp-uniform
+    const int n = min(nmax - m, size);
+    const int before = max(wait - m, 0);  // steps until the entry
+    float x0 = 1e9f, x1 = 1e9f, xe = 0.f, lo = 0.f;
+    u64 O = 0ull;
+    if (m < wait + nseg) {
+      const Around ar = around(s, park, c);
+      O = static_cast<u64>(static_cast<u32>(c.k[2])) << 32;
+      x0 = local_pos(ar.next[0], O);
+      x1 = local_pos(ar.next[1], O);
+      xe = local_pos(s.qx, O);
+      lo = m <= wait ? s.start : local_pos(ar.at, O);
+      lin = entry + static_cast<u32>(c.k[0]) * st[0] + static_cast<u32>(c.k[1]) * st[1] +
+            (static_cast<u32>(c.k[2]) - static_cast<u32>(before)) * st[2];
+    }
+    ac = lo;
+    float tx = static_cast<float>(1 - before), ty = x0, tz = x1, ly = 0.f, lz = 0.f;
+    int sl = static_cast<int>(lin);
+    int live = m - wait;  // the ray's segment of the next step
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+      const u32 at = static_cast<u32>(sl);
+      const float an = walk_step(tx, ty, tz, ly, lz, sl, static_cast<int>(st[2]), static_cast<int>(st[0]),
+                                 static_cast<int>(st[1]));
+      next_xy(ty, tz, ly, lz, s.r0, s.r1, x0, x1);
+      const float end = fminf(fmaxf(an, lo), xe);
+      const bool on = static_cast<u32>(live) < static_cast<u32>(nseg);
+#if DRR_CHECK_BOUNDS
+      // crossings closer than FP32 resolves may come in another order at the exit: a segment of no length
+      if (on && at >= nvox && end - ac > 1e-4f) atomicOr(&g_fault_word, kFaultBackproject);
+#endif
+      red_column_merged<kBpTileW>(gvol, on ? at : 0xffffffffu, gL * (end - ac), nvox, lane);
+      ac = end;
+      ++live;
     }
     m += n;
-    kx += static_cast<unsigned int>(cx);
-    ky += static_cast<unsigned int>(cy);
-    kz += static_cast<unsigned int>(cz);
-    // re-anchor at the last crossing taken: the current segment starts there
-    unsigned long long Onew = O;
-    if (kx) Onew = max(Onew, fix_at(ws->A0[0][t], ws->D[0][t], kx - 1u));
-    if (ky) Onew = max(Onew, fix_at(ws->A0[1][t], ws->D[1][t], ky - 1u));
-    if (kz) Onew = max(Onew, fix_at(ws->A0[2][t], ws->D[2][t], kz - 1u));
-    ac = 0.f;
-    O = Onew;
+    if (m > wait && m < wait + nseg) {
+      c.k[2] += static_cast<int>(tx) - 1;
+      c.k[0] += static_cast<int>(ly);
+      c.k[1] += static_cast<int>(lz);
+      // FP32 took the chunk's last crossings in another order
+      if (!around(s, park, c).ordered) c = counts_after(s, park, m - wait);
+    }
   }
 }
 
 // One warp's back-projection of its tile: every lane takes part in the walk,
 // with nseg = 0 where its pixel is outside the detector, its upstream gradient
 // is zero, the ray misses the volume or the geometry is not finite.
-__device__ __forceinline__ void backproject_tile_ray(const VolumeDev& vd, const PoseGeom& pg, int h, int w, bool active,
-                                                     float g, float* __restrict__ gvol, WalkScratch* ws, int lane) {
-  RaySetup r{};
-  int nseg = 0;
-  float gL = 0.f;
-  if (active && ray_setup(vd, pg, h, w, r) > 0) {
-    nseg = r.nseg;
-    gL = g * sqrtf(fmaf(r.d[2], r.d[2], fmaf(r.d[1], r.d[1], r.d[0] * r.d[0])));
-  }
-  walk_backproject(vd, r, nseg, gL, gvol, ws, lane);
+__device__ __forceinline__ void backproject_tile_ray(const VolumeDev& vd, const PoseGeom& pg, const GeomFF& gf, int h,
+                                                     int w, bool active, float g, float* __restrict__ gvol,
+                                                     FwdPark* park, int lane) {
+  SlabRay s;
+  const int rs = active ? slab_setup<kFwd>(vd, pg, gf, h, w, s, park) : 0;
+  const bool exact = rs > 0 && s.exact;
+  const u32 mask = __ballot_sync(0xffffffffu, exact);
+  if (mask) backproject_exact(vd, pg, mask, h, w, g, gvol);
+  if (rs <= 0 || exact) slab_idle(vd, s);
+  const int nseg = rs > 0 && !exact ? s.cnt[0] + s.cnt[1] + s.cnt[2] + 1 : 0;
+  walk_backproject(vd, s, park, nseg, nseg > 0 ? g * s.len * s.rg2 : 0.f, gvol, lane);
 }
 
 // The ray's outputs from its sums.
@@ -1808,14 +1887,15 @@ __device__ __forceinline__ void trace_tile(const VolumeDev& vd, const PoseGeom& 
 // when the pose changes.  Pose-gradient mode writes one partial sum of g . J
 // per tile, so the result does not depend on which warp took which tile.
 template <int MODE, int DT>
-__global__ void __launch_bounds__(kThreads, (MODE == kFwdJac || MODE == kPoseGrad || MODE == kGeoGrad) ? DRR_JAC_MINB
-                                                                                                : DRR_FWD_MINB)
+__global__ void __launch_bounds__(kThreads, MODE == kFwdJac || MODE == kPoseGrad || MODE == kGeoGrad ? DRR_JAC_MINB
+                                            : MODE == kBackproject                                   ? DRR_BP_MINB
+                                                                                                     : DRR_FWD_MINB)
     siddon_kernel(VolumeDev vd, DetDev det, const PoseGeom* __restrict__ pgs, int B, unsigned int* __restrict__ counter,
                   float* __restrict__ out, float* __restrict__ jac, const float* __restrict__ gin,
                   float* __restrict__ partials, float* __restrict__ gvol) {
   __shared__ PoseGeom spg[kThreads / 32];
   constexpr bool kBp = MODE == kBackproject;
-  constexpr bool kSlab = !std::is_same_v<typename ParkFor<MODE>::type, WalkScratch>;
+  constexpr bool kSlab = !std::is_same_v<typename ParkFor<MODE>::type, NoPark>;
   __shared__ typename ParkFor<MODE>::type ws;
   __shared__ GeomFF sgf[kSlab ? kThreads / 32 : 1];
   grid_dep_wait();
@@ -1853,7 +1933,7 @@ __global__ void __launch_bounds__(kThreads, (MODE == kFwdJac || MODE == kPoseGra
     float gsc = 0.f;
     if (valid && (MODE == kPoseGrad || MODE == kGeoGrad || kBp)) gsc = gin[b * npix + pix];
     if constexpr (kBp) {
-      backproject_tile_ray(vd, pg, h, w, valid && gsc != 0.f, gsc, gvol, &ws, lane);
+      backproject_tile_ray(vd, pg, sgf[warp], h, w, valid && gsc != 0.f, gsc, gvol, &ws, lane);
     } else if constexpr (MODE == kCount) {
       RaySetup rs;
       if (valid) reinterpret_cast<int*>(out)[b * npix + pix] = ray_setup(vd, pg, h, w, rs) > 0 ? rs.nseg : 0;
