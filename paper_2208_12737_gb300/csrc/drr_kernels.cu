@@ -907,15 +907,19 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
     // would lose more than FP32 keeps of them
     s.exact = exact || (s.cnt[0] > 0 && !(r20.x < 65536.f)) || (s.cnt[1] > 0 && !(r21.x < 65536.f)) || n[2] >= (1 << 23);
     if (s.exact) s.cnt[0] = s.cnt[1] = s.cnt[2] = 0;
-    s.qx = qx;
-    s.start = static_cast<float>(E[2]) * kTwoM32;
+    // a ray inside one slab (it clips a corner, or the volume is one slab thick) is
+    // measured from its entry: its lengths would carry 2^-24 of the slab otherwise,
+    // which may be a visible share of them
+    const u64 origin = s.cnt[2] == 0 ? E[2] : 0ull;
+    s.qx = qx - origin;
+    s.start = s.cnt[2] == 0 ? 0.f : static_cast<float>(E[2]) * kTwoM32;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const bool any = s.cnt[k] > 0;
       const float2 r = k == 0 ? r20 : r21;
       const u64 dx = ff_fix(any ? r : make_float2(0.f, 0.f)), dy = ff_fix40(k == 0 ? r02 : r12);
       park->dx[k][t] = dx;
-      park->x0[k][t] = any ? E[2] + (dx - mul_frac(E[k], dx)) : static_cast<u64>(1u << 30) << 32;  // none: beyond any exit
+      park->x0[k][t] = any ? E[2] - origin + (dx - mul_frac(E[k], dx)) : static_cast<u64>(1u << 30) << 32;  // none: beyond any exit
       park->dy[k][t] = dy;
       park->y0[k][t] = (static_cast<u64>(E[k]) << 8) + (dy - mul_frac(E[2], dy));
       (k == 0 ? s.r0 : s.r1) = any ? r.x : 0.f;
@@ -1157,7 +1161,7 @@ __device__ __forceinline__ void walk_forward(const VolumeDev& vd, const SlabRay&
       v = v1;
     }
     if (todo == 0) {  // the segment up to the exit
-      sink(q, fmaf(fix_to_float(static_cast<long long>(s.qx - O)) - ac, v, acc));
+      sink(q, fmaf(fix_to_float(static_cast<long long>(s.qx - ar.at)), v, acc));  // (no crossing: from the entry, 0)
       return;
     }
     sink(q, acc);
