@@ -67,3 +67,16 @@ def test_plain_fp32_baseline_is_close_but_unbounded(drr, case):
     # the textbook FP32 walk computes the same integral to FP32 accuracy, but its drift is not
     # held to the product tolerance
     assert np.median(err) < 1e-4 and err.max() < 1e-1, (np.median(err), err.max())
+
+
+@pytest.mark.parametrize("layout", ["x", "y", "z"])
+@pytest.mark.parametrize("storage", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (3, 5, 30), (2, 4, 31), (5, 3, 255), (4, 2, 300)])
+def test_ingest_row_lengths(drr, shape, storage, layout):
+    # rows at the edges of a warp's share; values that every storage holds exactly
+    vol_np = (np.arange(np.prod(shape)).reshape(shape) % 251 + 1).astype(np.float32)
+    det = inputs.Detector(2000.0, 2 * max(shape[:2]) + 3, 2 * max(shape) + 3, 1.0, 1.0)
+    poses_np = inputs.random_poses(2, seed=5, max_angle_deg=60, max_trans_mm=0.2)
+    E = drr.render(drr.Volume(vol_np, (1.0, 1.0, 1.0), storage=storage, layout=layout), det, torch.from_numpy(poses_np).cuda())
+    ref = oracle.render(ovol(vol_np, (1.0, 1.0, 1.0)), odet(det), poses_np)
+    assert ref.max() > 0 and rel_err(E.cpu().numpy(), ref).max() < FP32_TOL
