@@ -91,6 +91,9 @@ __global__ void __cluster_dims__(kZCluster, 1, 1) __launch_bounds__(kZThreads)
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = static_cast<int>(cluster.block_rank()), pair = static_cast<int>(blockIdx.x / kZCluster);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  // a block's shared memory may be written by another only once that block runs:
+  // every block says so here, and the first remote write below waits for all
+  cluster.barrier_arrive();
   __shared__ double part[kZSums][kZThreads];
   __shared__ float range[kZThreads / 32];
   __shared__ double rows[kZCluster][kZSums + 1];  // every block's sums and largest magnitude
@@ -142,6 +145,7 @@ __global__ void __cluster_dims__(kZCluster, 1, 1) __launch_bounds__(kZThreads)
     const bool any = __any_sync(0xffffffffu, largest != 0.f);
     if (lane == 0) range[warp] = any ? 1.f : 0.f;
     __syncthreads();
+    if (!wide) cluster.barrier_wait();  // (the second pass: the sync at the end of the first)
     if (warp < kZSums) {  // warp k: the block's sum k, in a fixed order
       double x = 0.0;
 #pragma unroll
