@@ -599,7 +599,8 @@ enum ParkSlot : int {
   kPkF0 = 6,      // alpha from the entry to the first crossing of slots 0, 1 (2)
   kPkRg = 8,      // alpha per plane of slots 0, 1 (2)
   kPkSpan = 10,   // alpha_max - alpha_min
-  kPkCount = 11
+  kPkMm = 11,     // path length of a slab, a float-float (2)
+  kPkCount = 13
 };
 struct Park {
   float v[kPkCount][kThreads];
@@ -621,8 +622,10 @@ struct SlabRay {
   int i0[3];       // entry voxel index per slot, counted in the ray's direction
   int off;         // element offset of the entry voxel (padded layout)
   int step[3];     // signed element stride per slot
-  int ax0, ax1, ax2;  // real axis of each slot
-  int ea, xa;      // axis of the entry / exit plane, -1 when clamped to alpha = 0 / 1
+  u32 axes;        // 2 bits each: real axis of slots 0, 1, 2; slot of the entry / exit plane, 3 when clamped to alpha = 0 / 1
+  __device__ __forceinline__ int axis(int slot) const { return (axes >> (2 * slot)) & 3u; }
+  __device__ __forceinline__ int entry_slot() const { return (axes >> 6) & 3u; }
+  __device__ __forceinline__ int exit_slot() const { return (axes >> 8) & 3u; }
   u64 Y, Z;        // q_0, q_1 at dominant crossing 0 and their step per dominant crossing
   u32 dy, dz;
   u64 mX, mdX;     // slot 0's crossing 0: q_2 and q_1 (both + t0) and their steps
@@ -633,13 +636,13 @@ struct SlabRay {
   u32 t0, t1;      // rounding bounds (and biases) of the minor loops' coordinates
   float w1;        // 1 - q_2 at the entry: the first slab's share inside the ray
   float rest;      // share of the last slab beyond the exit
-  float rg2;       // alpha per dominant plane
   bool exact;      // to be summed by exact_rays
   // the forward walk only
   u64 qx;          // q_2 at the exit
   float start;     // q_2 at the entry
   float r0, r1;    // slabs per plane of slots 0, 1
   float len;       // |p - s| in mm
+  float rg2;       // alpha per dominant plane
 };
 
 // A lane without a ray to walk takes part with no crossings.
@@ -681,6 +684,40 @@ __device__ __forceinline__ float2 ff_rcp(float2 a) {  // 1e-30 < |a| < 1e30
   const float r = __frcp_rn(a.x);
   const float e = __fmaf_rn(-a.y, r, __fmaf_rn(-a.x, r, 1.f));
   return ff_norm(r, __fmul_rn(r, e));
+}
+// A sum kept as value + error: exact but for the rounding of the error.
+struct Sum2 {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float2 r = ff_sum(s, x);
+    s = r.x;
+    e = __fadd_rn(e, r.y);
+  }
+  __device__ __forceinline__ void add(Sum2 x) {
+    add(x.s);
+    e = __fadd_rn(e, x.e);
+  }
+  __device__ __forceinline__ void add_product(float x, float y) {
+    const float p = __fmul_rn(x, y);
+    add(p);
+    e = __fadd_rn(e, __fmaf_rn(x, y, -p));
+  }
+  // (an infinite or NaN s is the plain sum's; its error is NaN)
+  __device__ __forceinline__ float value() const { return isfinite(s) ? __fadd_rn(s, e) : s; }
+};
+__device__ __forceinline__ float2 ff_sqr(float2 a) {
+  const float p = __fmul_rn(a.x, a.x);
+  return ff_norm(p, __fmaf_rn(__fadd_rn(a.x, a.x), a.y, __fmaf_rn(a.x, a.x, -p)));
+}
+__device__ __forceinline__ float2 ff_sqrt(float2 a) {  // 1e-30 < a < 1e30
+  const float r = __fsqrt_rn(a.x);
+  return ff_norm(r, __fmul_rn(__fadd_rn(__fmaf_rn(-r, r, a.x), a.y), __fmul_rn(0.5f, __frcp_rn(r))));
+}
+// a times c, rounded once (to its last bit or so).
+__device__ __forceinline__ float ff_scaled(const Sum2& a, float2 c) {
+  const float p = __fmul_rn(a.s, c.x);
+  if (!isfinite(p)) return p;
+  return __fadd_rn(p, __fadd_rn(__fmaf_rn(a.s, c.x, -p), __fmaf_rn(a.s, c.y, __fmul_rn(a.e, c.x))));
 }
 // x as the unevaluated sum of two FP32 numbers.
 __device__ __forceinline__ float2 ff_from(double x) {
@@ -801,11 +838,8 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
   const int p = a2 == 0 ? 1 : 0, q = a2 == 2 ? 1 : 2;
   const bool pq = !more(pick3(q, ag[0], ag[1], ag[2]), pick3(p, ag[0], ag[1], ag[2]));
   const int ax[3] = {pq ? p : q, pq ? q : p, a2};
-  s.ax0 = ax[0];
-  s.ax1 = ax[1];
-  s.ax2 = ax[2];
-  s.ea = ea;
-  s.xa = xa;
+  const auto slot_of = [&](int a) { return a < 0 ? 3u : (a == ax[0] ? 0u : (a == ax[1] ? 1u : 2u)); };
+  s.axes = static_cast<u32>(ax[0] | ax[1] << 2 | ax[2] << 4) | slot_of(ea) << 6 | slot_of(xa) << 8;
   float2 sg[3], sr[3], U[3], N[3];  // direction, its reciprocal, source and far face (in the ray's direction), per slot
   int n[3];
   bool up[3];
@@ -968,6 +1002,13 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
     park->v[kPkRg][t] = sr[0].x;
     park->v[kPkRg + 1][t] = sr[1].x;
     park->v[kPkSpan][t] = fix_float(len) * sr[2].x;
+    // the path length of a slab as float-float: the roundings of an FP32 product of
+    // length and alpha per slab were a third of a pixel's error
+    const auto side = [&](int k) { return make_float2(pick3(ax[k], vd.delta[0], vd.delta[1], vd.delta[2]), 0.f); };
+    const float2 sq = ff_add(ff_add(ff_sqr(ff_mul(r02, side(0))), ff_sqr(ff_mul(r12, side(1)))), ff_sqr(side(2)));
+    const float2 mm = sq.x > 1e-24f && sq.x < 1e30f ? ff_sqrt(sq) : make_float2(L * sr[2].x, 0.f);
+    park->v[kPkMm][t] = mm.x;
+    park->v[kPkMm + 1][t] = mm.y;
   }
   return 1;
 }
@@ -1201,7 +1242,10 @@ __device__ __forceinline__ int piece_start(const Pieces& pc, int p, int cnt) {
 }
 
 // Pieces [p0, p1) of the sum of the voxels entered at dominant crossings; piece
-// p's sum goes to sink(p, sum).
+// p's sum goes to sink(p, sum).  A block of kSlabUnroll voxels is added as a tree:
+// a homogeneous tissue has few voxel values, and a running FP32 sum rounds each of
+// them the same way on every ray, a common error of a DRR's pixels that does not
+// average out of their sums (the pose gradient).
 template <int DT, class Sink>
 __device__ __forceinline__ void dominant_loop(const VolumeDev& vd, const SlabRay& s, const Pieces& pc, int p0, int p1,
                                               Sink sink) {
@@ -1215,20 +1259,37 @@ __device__ __forceinline__ void dominant_loop(const VolumeDev& vd, const SlabRay
   for (int p = p0; p < p1; ++p) {
     const int end = piece_start(pc, p + 1, s.cnt[2]);
     float S = 0.f;
-#pragma unroll kSlabUnroll
-    for (; m < end; ++m) {
-      S += gather<DT>(vd, off);
-      fy += s.dy;
-      fz += s.dz;
-      off += (fy < s.dy ? st0 : st) + (fz < s.dz ? s1 : 0);
+    const auto block = [&](auto whole) {
+      float v[kSlabUnroll];
+#pragma unroll
+      for (int j = 0; j < kSlabUnroll; ++j) {
+        v[j] = 0.f;
+        if (whole || m + j < end) {
+          v[j] = gather<DT>(vd, off);
+          fy += s.dy;
+          fz += s.dz;
+          off += (fy < s.dy ? st0 : st) + (fz < s.dz ? s1 : 0);
+        }
+      }
+#pragma unroll
+      for (int o = kSlabUnroll / 2; o > 0; o >>= 1) {
+#pragma unroll
+        for (int j = 0; j < o; ++j) v[j] += v[j + o];
+      }
+      S += v[0];
+    };
+    for (; m + kSlabUnroll <= end; m += kSlabUnroll) block(std::true_type{});
+    if (m < end) {
+      block(std::false_type{});
+      m = end;
     }
     sink(p, S);
   }
 }
 
-// Sums over one minor axis' crossings, w = V after - V before: g = sum w,
-// c = sum w f (f: biased fraction of the slab at the crossing, times 2^32), h =
-// sum w k (Jacobian modes); near: the smallest biased fraction.
+// Sums over one minor axis' crossings of a piece, w = V after - V before: g = sum
+// w, c = sum w f (f: biased fraction of the slab at the crossing, times 2^32), h =
+// sum w k (k from the piece's first crossing); near: the smallest biased fraction.
 struct MinorSums {
   float g, c, h;
   u32 near;
@@ -1258,7 +1319,7 @@ struct MinorSums {
   }
 #define DRR_MINOR_PIECES(CNT, ADVANCE)                                 \
   _Pragma("unroll 1") for (int p = p0; p < p1; ++p) {                  \
-    const int end = piece_start(pc, p + 1, CNT), k0 = k;               \
+    const int end = piece_start(pc, p + 1, CNT);                       \
     MinorSums r{0.f, 0.f, 0.f, 0xffffffffu};                           \
     float kf = 0.f;                                                    \
     for (; k + kU <= end; k += kU) DRR_MINOR_BLOCK(true, ADVANCE)      \
@@ -1266,7 +1327,6 @@ struct MinorSums {
       DRR_MINOR_BLOCK(k + j < end, ADVANCE)                            \
       k = end;                                                         \
     }                                                                  \
-    r.h = fmaf(static_cast<float>(k0), r.g, r.h);                      \
     sink(p, r);                                                        \
   }
 
@@ -1310,30 +1370,29 @@ __device__ __forceinline__ void least_loop(const VolumeDev& vd, const SlabRay& s
 #undef DRR_MINOR_PIECES
 #undef DRR_MINOR_BLOCK
 
-// Whole-ray sums of the pieces, added in piece order.
-struct SlabTotals {
-  float S, g0, c0, h0, g1, c1, h1;
-  __device__ __forceinline__ void add(int slot, const MinorSums& r) {
-    if (slot == 2) {
-      S += r.g;
-    } else if (slot == 0) {
-      g0 += r.g;
-      c0 += r.c;
-      h0 += r.h;
-    } else {
-      g1 += r.g;
-      c1 += r.c;
-      h1 += r.h;
-    }
+// Whole-ray sums of one minor axis' pieces, added in piece order as value + error.
+struct MinorTotals {
+  Sum2 g, c, h;
+  // first: the piece's first crossing (h counts from the ray's)
+  __device__ __forceinline__ void add(float pg, float pc, float ph, int first) {
+    g.add(pg);
+    c.add(pc);
+    h.add(ph);
+    h.add_product(static_cast<float>(first), pg);
   }
+  __device__ __forceinline__ float3 value() const { return make_float3(g.value(), c.value(), h.value()); }
+};
+struct SlabTotals {
+  Sum2 S;
+  float3 minor[2];  // g, c, h of slots 0 and 1
 };
 
-// What the ray's end takes from the walk: F in alpha units; with the Jacobian
+// What the ray's end takes from the walk: E; with the Jacobian
 // the per-axis crossing sums G = sum w, A = sum w alpha (w = V before - V
 // after, alpha from the entry; A of the dominant axis is not used), and the
 // parts of the clamped end points (Gc, Ac), which belong to no axis.
 struct JacSums {
-  float F, G[3], A[3], Gc, Ac;
+  float E, G[3], A[3], Gc, Ac;
   int dom;
 };
 // exact_rays' answer: the sums and the ray's entry in world coordinates, amin
@@ -1431,7 +1490,7 @@ __device__ __noinline__ void exact_rays(const VolumeDev& vd, const PoseGeom& pg,
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) F += __shfl_xor_sync(kAll, F, o);
-      q.F = F * r.unit;
+      q.E = F * r.unit * sqrtf(fmaf(r.d[2], r.d[2], fmaf(r.d[1], r.d[1], r.d[0] * r.d[0])));
       const float ex = static_cast<float>(kExitUnits);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
@@ -1463,10 +1522,14 @@ __device__ __forceinline__ void slab_finish(const VolumeDev& vd, const PoseGeom&
   const float v1 = gather<DT>(vd, s.off);
   const float vl = gather<DT>(vd, s.off + s.cnt[0] * s.step[0] + s.cnt[1] * s.step[1] + s.cnt[2] * s.step[2]);
   // sum w (1 - f), f the unbiased fraction
+  const float g0 = T.minor[0].x, g1 = T.minor[1].x;
   const float b0 = static_cast<float>(s.t0) * kTwoM32, b1 = static_cast<float>(s.t1) * kTwoM32;
-  const float m0 = fmaf(-kTwoM32, T.c0, fmaf(b0, T.g0, T.g0));
-  const float m1 = fmaf(-kTwoM32, T.c1, fmaf(b1, T.g1, T.g1));
-  const float F = fmaf(-s.rest, vl, fmaf(v1, s.w1, T.S + (m0 + m1)));
+  Sum2 sum = T.S;
+  sum.add(fmaf(-kTwoM32, T.minor[0].y, fmaf(b0, g0, g0)));
+  sum.add(fmaf(-kTwoM32, T.minor[1].y, fmaf(b1, g1, g1)));
+  sum.add_product(v1, s.w1);
+  sum.add_product(-s.rest, vl);
+  const float F = sum.value();
   // a sum that is not finite (an infinite or NaN voxel) is taken segment by segment instead
   exact = live && (exact || !(fabsf(F) <= 3.0e38f));
   const u32 mask = __ballot_sync(0xffffffffu, exact);
@@ -1485,24 +1548,25 @@ __device__ __forceinline__ void slab_finish(const VolumeDev& vd, const PoseGeom&
       return;
     }
   }
-  out.F = F * s.rg2;
-  float G0 = -T.g0, G1 = -T.g1;
-  float A0 = -fmaf(park->v[kPkRg][t], T.h0, park->v[kPkF0][t] * T.g0);
-  float A1 = -fmaf(park->v[kPkRg + 1][t], T.h1, park->v[kPkF0 + 1][t] * T.g1);
+  out.E = ff_scaled(sum, make_float2(park->v[kPkMm][t], park->v[kPkMm + 1][t]));
+  float G0 = -g0, G1 = -g1;
+  float A0 = -fmaf(park->v[kPkRg][t], T.minor[0].z, park->v[kPkF0][t] * g0);
+  float A1 = -fmaf(park->v[kPkRg + 1][t], T.minor[1].z, park->v[kPkF0 + 1][t] * g1);
   const float ex = vl * park->v[kPkSpan][t];
   // entry crossing: weight 0 - V first at alpha 0; exit crossing: V last - 0 at the span
   float Gc = 0.f, Ac = 0.f;
-  if (s.ea < 0) Gc -= v1;
-  if (s.ea == s.ax0) G0 -= v1;
-  if (s.ea == s.ax1) G1 -= v1;
-  if (s.xa < 0) { Gc += vl; Ac = ex; }
-  if (s.xa == s.ax0) { G0 += vl; A0 += ex; }
-  if (s.xa == s.ax1) { G1 += vl; A1 += ex; }
-  out.dom = s.ax2;
+  const int es = s.entry_slot(), xs = s.exit_slot(), ax0 = s.axis(0), ax1 = s.axis(1);
+  if (es == 3) Gc -= v1;
+  if (es == 0) G0 -= v1;
+  if (es == 1) G1 -= v1;
+  if (xs == 3) { Gc += vl; Ac = ex; }
+  if (xs == 0) { G0 += vl; A0 += ex; }
+  if (xs == 1) { G1 += vl; A1 += ex; }
+  out.dom = s.axis(2);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {  // static indices: the arrays stay in registers
-    out.G[a] = a == s.ax0 ? G0 : (a == s.ax1 ? G1 : -(G0 + G1 + Gc));  // sum of all crossing weights is 0
-    out.A[a] = a == s.ax0 ? A0 : (a == s.ax1 ? A1 : 0.f);              // the dominant axis is handled through R
+    out.G[a] = a == ax0 ? G0 : (a == ax1 ? G1 : -(G0 + G1 + Gc));  // sum of all crossing weights is 0
+    out.A[a] = a == ax0 ? A0 : (a == ax1 ? A1 : 0.f);              // the dominant axis is handled through R
   }
   out.Gc = Gc;
   out.Ac = Ac;
@@ -1521,7 +1585,7 @@ __device__ __forceinline__ void slab_finish(const VolumeDev& vd, const PoseGeom&
 __device__ __forceinline__ void ray_world_grads(const float d[3], const JacSums& s, float gt[3], float q[3]) {
   const float L2 = fmaf(d[2], d[2], fmaf(d[1], d[1], d[0] * d[0]));
   const float L = sqrtf(L2);
-  const float F = s.F;
+  const float F = s.E / L;  // in units of alpha
   float R = s.Ac;  // position sums relative to the entry
 #pragma unroll
   for (int a = 0; a < 3; ++a)
@@ -1717,7 +1781,7 @@ __device__ __forceinline__ void walk_backproject(const VolumeDev& vd, const Slab
   u32 st[3], entry = 0u;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const int ax = k == 0 ? s.ax0 : (k == 1 ? s.ax1 : s.ax2);
+    const int ax = s.axis(k);
     const u32 u = pick3(ax, 1u, nx, nxy);
     const bool up = s.step[k] > 0;
     entry += u * static_cast<u32>(up ? s.i0[k] : pick3(ax, vd.n[0], vd.n[1], vd.n[2]) - 1 - s.i0[k]);
@@ -1804,32 +1868,13 @@ __device__ __forceinline__ void ray_outputs(const VolumeDev& vd, const PoseGeom&
                                             const Park* park, RayResult& res) {
   const int t = threadIdx.x;
   const float d[3] = {park->v[kPkD][t], park->v[kPkD + 1][t], park->v[kPkD + 2][t]};
-  res.F = q.F * sqrtf(fmaf(d[2], d[2], fmaf(d[1], d[1], d[0] * d[0]))) * vd.out_scale;
+  res.F = q.E * vd.out_scale;
   if (MODE != kGeoGrad) {
     const float e[3] = {park->v[kPkE][t], park->v[kPkE + 1][t], park->v[kPkE + 2][t]};
     pose_jacobian(d, q, pg, e, h, w, vd.out_scale, res.J);
   } else {
     geometry_jacobian(d, q, pg, park->v[kPkE + 1][t], park->v[kPkE][t], h, w, vd.out_scale, res.J);
   }
-}
-
-// Pieces [p0, p1) of the ray's three loops, each piece's sums to sink(p, slot,
-// sums) (slot 2: g alone); true if a pair of crossings in them was too close to
-// order.
-template <int DT, class Sink>
-__device__ __forceinline__ bool walk_pieces(const VolumeDev& vd, const SlabRay& s, const Plan& pl, int p0, int p1,
-                                            Sink sink) {
-  bool near = false;
-  least_loop<DT>(vd, s, pl.slot[1], p0, p1, [&](int p, const MinorSums& r) {
-    near |= r.near < 2u * s.t1;
-    sink(p, 1, r);
-  });
-  middle_loop<DT>(vd, s, pl.slot[0], p0, p1, [&](int p, const MinorSums& r) {
-    near |= r.near < 2u * s.t0;
-    sink(p, 0, r);
-  });
-  dominant_loop<DT>(vd, s, pl.slot[2], p0, p1, [&](int p, float S) { sink(p, 2, MinorSums{S, 0.f, 0.f, 0u}); });
-  return near;
 }
 
 // The DRR value from the sum of a ray's chunks (all 32 lanes call; rs as
@@ -1839,13 +1884,13 @@ __device__ __forceinline__ float forward_finish(const VolumeDev& vd, const PoseG
                                                 const SlabRay& s, float F) {
   const bool exact = rs > 0 && (s.exact || !(fabsf(F) <= 3.0e38f));  // a voxel that is not finite: segment by segment
   const u32 mask = __ballot_sync(0xffffffffu, exact);
-  F *= s.rg2;
+  F *= s.rg2 * s.len;
   if (mask) {
     ExactRay x;
     exact_rays<DT>(vd, pg, mask, h, w, &x);
-    if (exact) F = x.q.F;
+    if (exact) F = x.q.E;
   }
-  return rs < 0 ? __int_as_float(0x7fffffff) : (rs > 0 ? F * s.len * vd.out_scale : 0.f);
+  return rs < 0 ? __int_as_float(0x7fffffff) : (rs > 0 ? F * vd.out_scale : 0.f);
 }
 
 // The rays of one warp tile (all 32 lanes call; a lane outside the detector
@@ -1869,9 +1914,25 @@ __device__ __forceinline__ void trace_tile(const VolumeDev& vd, const PoseGeom& 
     const int rs = valid ? slab_setup<MODE>(vd, pg, gf, h, w, s, park) : 0;
     if (rs <= 0) slab_idle(vd, s);
     bool exact = s.exact;
-    SlabTotals T{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    SlabTotals T;
     const Plan pl = plan_pieces(s);
-    exact |= walk_pieces<DT>(vd, s, pl, 0, pl.np, [&](int, int slot, const MinorSums& r) { T.add(slot, r); });
+    {
+      MinorTotals m;
+      least_loop<DT>(vd, s, pl.slot[1], 0, pl.np, [&](int p, const MinorSums& r) {
+        exact |= r.near < 2u * s.t1;
+        m.add(r.g, r.c, r.h, piece_start(pl.slot[1], p, s.cnt[1]));
+      });
+      T.minor[1] = m.value();
+    }
+    {
+      MinorTotals m;
+      middle_loop<DT>(vd, s, pl.slot[0], 0, pl.np, [&](int p, const MinorSums& r) {
+        exact |= r.near < 2u * s.t0;
+        m.add(r.g, r.c, r.h, piece_start(pl.slot[0], p, s.cnt[0]));
+      });
+      T.minor[0] = m.value();
+    }
+    dominant_loop<DT>(vd, s, pl.slot[2], 0, pl.np, [&](int, float S) { T.S.add(S); });
     JacSums q;
     slab_finish<MODE, DT>(vd, pg, h, w, rs > 0, s, T, exact, park, q);
     if (rs < 0) {  // non-finite geometry (e.g. a NaN pose): NaN out, no walk
@@ -2039,11 +2100,16 @@ __global__ void __launch_bounds__(32 * K) siddon_split_kernel(VolumeDev vd, DetD
       bool exact = s.exact;
       const Plan pl = plan_pieces(s);
       // this warp's share of the pieces
-      exact |= walk_pieces<DT>(vd, s, pl, pl.np * warp / K, pl.np * (warp + 1) / K,
-                                     [&](int p, int slot, const MinorSums& r) {
-                                       if (slot == 2) piece[p].S[lane] = r.g;
-                                       else piece[p].minor[slot][lane] = make_float3(r.g, r.c, r.h);
-                                     });
+      const int p0 = pl.np * warp / K, p1 = pl.np * (warp + 1) / K;
+      least_loop<DT>(vd, s, pl.slot[1], p0, p1, [&](int p, const MinorSums& r) {
+        exact |= r.near < 2u * s.t1;
+        piece[p].minor[1][lane] = make_float3(r.g, r.c, r.h);
+      });
+      middle_loop<DT>(vd, s, pl.slot[0], p0, p1, [&](int p, const MinorSums& r) {
+        exact |= r.near < 2u * s.t0;
+        piece[p].minor[0][lane] = make_float3(r.g, r.c, r.h);
+      });
+      dominant_loop<DT>(vd, s, pl.slot[2], p0, p1, [&](int p, float S) { piece[p].S[lane] = S; });
       const unsigned int ex = __ballot_sync(0xffffffffu, exact);
       if (lane == 0) exact_s[warp] = ex;
       __syncthreads();
@@ -2051,15 +2117,18 @@ __global__ void __launch_bounds__(32 * K) siddon_split_kernel(VolumeDev vd, DetD
         r.F = rs < 0 ? __int_as_float(0x7fffffff) : 0.f;
 #pragma unroll
         for (int k = 0; k < 6; ++k) r.J[k] = r.F;
-        SlabTotals T{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        SlabTotals T;
+        MinorTotals m[2];
         for (int p = 0; p < pl.np; ++p) {
 #pragma unroll
           for (int k = 0; k < 2; ++k) {
             const float3 q = piece[p].minor[k][lane];
-            T.add(k, MinorSums{q.x, q.y, q.z, 0u});
+            m[k].add(q.x, q.y, q.z, piece_start(pl.slot[k], p, s.cnt[k]));
           }
-          T.add(2, MinorSums{piece[p].S[lane], 0.f, 0.f, 0u});
+          T.S.add(piece[p].S[lane]);
         }
+        T.minor[0] = m[0].value();
+        T.minor[1] = m[1].value();
         unsigned int any = 0u;
 #pragma unroll
         for (int k = 0; k < K; ++k) any |= exact_s[k];
