@@ -704,6 +704,15 @@ struct Sum2 {
   }
   // (an infinite or NaN s is the plain sum's; its error is NaN)
   __device__ __forceinline__ float value() const { return isfinite(s) ? __fadd_rn(s, e) : s; }
+  __device__ __forceinline__ double value64() const {
+    return isfinite(s) ? static_cast<double>(s) + static_cast<double>(e) : static_cast<double>(s);
+  }
+  // Total over the warp, the same in every lane (a fixed butterfly).
+  __device__ __forceinline__ void warp_sum() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      add(Sum2{__shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, e, o)});
+  }
 };
 __device__ __forceinline__ float2 ff_sqr(float2 a) {
   const float p = __fmul_rn(a.x, a.x);
@@ -2151,10 +2160,11 @@ __global__ void __launch_bounds__(32 * K) siddon_split_kernel(VolumeDev vd, DetD
 // Pose gradient from a stored Jacobian in one launch (Sec. 2.4, chain rule:
 // dL/d eta = sum over pixels of dL/dE * dE/d eta).  One thread-block cluster
 // per pose: block r of the cluster sums g * J over the r-th of kJacCluster
-// contiguous shares of the pose's pixels (in FP32: FP64 arithmetic is narrow
-// on this GPU), writes its six sums into a row of block 0's shared memory
-// through the cluster's distributed shared memory, and block 0 adds the rows
-// in rank order in FP64.  Every sum has a fixed order, so the result is
+// contiguous shares of the pose's pixels (as FP32 value + error with exact
+// products: FP64 arithmetic is narrow on this GPU, and where the sum cancels to a
+// small component, plain FP32 totals left 1e-8 of sum |g J| in it), writes its six
+// sums into a row of block 0's shared memory through the cluster's distributed
+// shared memory, and block 0 adds the rows in rank order in FP64.  Every sum has a fixed order, so the result is
 // bitwise reproducible, and no partial sums leave the chip.
 constexpr int kJacCluster = 8;  // blocks per pose (the portable cluster size)
 #ifndef DRR_JAC_THREADS
@@ -2165,14 +2175,14 @@ constexpr int kJacCluster = 8;  // blocks per pose (the portable cluster size)
 // 16-pose batch took two waves, 16.8 us).
 constexpr int kJacThreads = DRR_JAC_THREADS;
 
-__device__ __forceinline__ void jac_fma4(float c[6], const float4 gv, const float* __restrict__ jb, int npix, int i) {
+__device__ __forceinline__ void jac_fma4(Sum2 c[6], const float4 gv, const float* __restrict__ jb, int npix, int i) {
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const float4 jv = __ldcs(reinterpret_cast<const float4*>(jb + static_cast<size_t>(k) * npix) + i);
-    c[k] = fmaf(gv.x, jv.x, c[k]);
-    c[k] = fmaf(gv.y, jv.y, c[k]);
-    c[k] = fmaf(gv.z, jv.z, c[k]);
-    c[k] = fmaf(gv.w, jv.w, c[k]);
+    c[k].add_product(gv.x, jv.x);
+    c[k].add_product(gv.y, jv.y);
+    c[k].add_product(gv.z, jv.z);
+    c[k].add_product(gv.w, jv.w);
   }
 }
 
@@ -2180,7 +2190,7 @@ __global__ void __cluster_dims__(kJacCluster, 1, 1) __launch_bounds__(kJacThread
     jac_grad_kernel(const float* __restrict__ gin, const float* __restrict__ jac, int npix, int vec,
                     float* __restrict__ grad) {
   static_assert(kJacThreads % 32 == 0 && kJacThreads <= 32 * 32, "the block sum takes one warp sum per lane");
-  __shared__ float wsum[kJacThreads / 32][6];
+  __shared__ float2 wsum[kJacThreads / 32][6];
   __shared__ double rows[kJacCluster][6];  // filled in block 0 only
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
@@ -2191,7 +2201,7 @@ __global__ void __cluster_dims__(kJacCluster, 1, 1) __launch_bounds__(kJacThread
   grid_dep_release();
   const float* gb = gin + static_cast<size_t>(b) * npix;
   const float* jb = jac + static_cast<size_t>(b) * 6 * npix;
-  float c[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  Sum2 c[6];
   if (vec) {  // npix % 4 == 0 and 16-byte aligned planes: float4 loads
     const int nv = npix >> 2;
     const int lo = static_cast<int>(static_cast<int64_t>(nv) * rank / kJacCluster);
@@ -2202,39 +2212,44 @@ __global__ void __cluster_dims__(kJacCluster, 1, 1) __launch_bounds__(kJacThread
   } else {
     const int lo = static_cast<int>(static_cast<int64_t>(npix) * rank / kJacCluster);
     const int hi = static_cast<int>(static_cast<int64_t>(npix) * (rank + 1) / kJacCluster);
+    constexpr int kU = 4;  // pixels in flight per thread (154 us for 4 poses of 509x451 with one, 42 with FP32 sums)
 #pragma unroll 1
-    for (int p = lo + threadIdx.x; p < hi; p += kJacThreads) {
-      const float gv = __ldcs(gb + p);
+    for (int p = lo + threadIdx.x; p < hi; p += kU * kJacThreads) {
+      float gv[kU], jv[kU][6];
 #pragma unroll
-      for (int k = 0; k < 6; ++k) c[k] = fmaf(gv, __ldcs(jb + static_cast<size_t>(k) * npix + p), c[k]);
+      for (int u = 0; u < kU; ++u) {
+        const int q = p + u * kJacThreads;
+        gv[u] = q < hi ? __ldcs(gb + q) : 0.f;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) jv[u][k] = q < hi ? __ldcs(jb + static_cast<size_t>(k) * npix + q) : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) c[k].add_product(gv[u], jv[u][k]);
+      }
     }
   }
 #pragma unroll
-  for (int k = 0; k < 6; ++k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c[k] += __shfl_xor_sync(0xffffffffu, c[k], o);
-  }
+  for (int k = 0; k < 6; ++k) c[k].warp_sum();
   if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) wsum[warp][k] = c[k];
+    for (int k = 0; k < 6; ++k) wsum[warp][k] = make_float2(c[k].s, c[k].e);
   }
   __syncthreads();
   // every block of the cluster is running (its shared memory exists) before any
   // block writes into block 0's
   cluster.sync();
   if (warp == 0) {  // lane q holds warp q's sums; a fixed butterfly adds them
-    float t[6];
+    double mine = 0.0;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      t[k] = lane < kJacThreads / 32 ? wsum[lane][k] : 0.f;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+      Sum2 t;
+      if (lane < kJacThreads / 32) t = Sum2{wsum[lane][k].x, wsum[lane][k].y};
+      t.warp_sum();
+      if (lane == k) mine = t.value64();
     }
-    float mine = t[0];
-#pragma unroll
-    for (int k = 1; k < 6; ++k)
-      if (lane == k) mine = t[k];
-    if (lane < 6) cluster.map_shared_rank(&rows[0][0], 0)[rank * 6 + lane] = static_cast<double>(mine);
+    if (lane < 6) cluster.map_shared_rank(&rows[0][0], 0)[rank * 6 + lane] = mine;
   }
   cluster.sync();  // rows complete; no block exits while its row is still being written
   if (rank == 0 && threadIdx.x < 6) {

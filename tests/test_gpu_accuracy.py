@@ -35,3 +35,35 @@ def test_jacobian_renders_sum_their_voxels_to_the_last_bits(drr):
     through = ref > 0.3 * ref.max()
     err = (E.cpu().numpy().astype(np.float64) - ref)[through] / ref[through]
     assert through.mean() > 0.5 and np.sqrt((err**2).mean()) < 5e-8, np.sqrt((err**2).mean())
+
+
+@pytest.mark.parametrize("H, W", [(64, 80), (61, 37), (1, 1), (3, 5), (211, 193)])
+def test_stored_jacobian_gradient_of_cancelling_sums(drr, H, W):
+    # the sum over pixels cancels to ~1e-4 of its terms; value + error sums lose less than
+    # 2^-40 of the terms, and the result is rounded once
+    rng = np.random.default_rng(H)
+    B, n = 2, H * W
+    J = rng.normal(size=(B, 6, n)).astype(np.float32)
+    g = rng.normal(size=(B, n)).astype(np.float32)
+    h = n // 2
+    g[:, h:2 * h] = -g[:, :h]
+    J[:, :, h:2 * h] = J[:, :, :h] * np.float32(1.0001)
+    vol = drr.Volume(np.ones((4, 4, 4), np.float32), (1.0, 1.0, 1.0))
+    P = torch.zeros((B, 6), device="cuda")
+    G = drr.render_backward(vol, inputs.Detector(100.0, H, W, 1.0, 1.0), P, torch.from_numpy(g.reshape(B, H, W)).cuda(),
+                            jac=torch.from_numpy(J.reshape(B, 6, H, W)).cuda()).cpu().numpy()
+    terms = J.astype(np.float64) * g[:, None]
+    ref = terms.sum(2)
+    assert (np.abs(G - ref) <= 2.0**-24 * np.abs(ref) + 2.0**-40 * np.abs(terms).sum(2)).all()
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf])
+def test_stored_jacobian_gradient_stays_infinite(drr, bad):
+    H, W = 40, 37
+    J = np.ones((1, 6, H, W), np.float32)
+    g = np.ones((1, H, W), np.float32)
+    g[0, 20, 11] = bad
+    vol = drr.Volume(np.ones((4, 4, 4), np.float32), (1.0, 1.0, 1.0))
+    G = drr.render_backward(vol, inputs.Detector(100.0, H, W, 1.0, 1.0), torch.zeros((1, 6), device="cuda"),
+                            torch.from_numpy(g).cuda(), jac=torch.from_numpy(J).cuda())
+    np.testing.assert_array_equal(G.cpu().numpy(), np.full((1, 6), bad, np.float32))
