@@ -3,6 +3,7 @@
 // moving DRR and a fixed image): the ZNCC loss with its image gradient, and an
 // Adam step on the pose parameters.
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include <cooperative_groups.h>
@@ -211,21 +212,22 @@ __global__ void __cluster_dims__(kZCluster, 1, 1) __launch_bounds__(kZThreads)
 }
 
 // Adam on the six pose parameters of each of B poses (rotations and
-// translations have separate step sizes, Sec. 3.2 uses separate rates too).
+// translations have separate step sizes, Sec. 3.2 uses separate rates too).  In
+// FP64, as the rounding of the quotient alone may move an FP32 pose by its last
+// bit, which re-orders some rays' crossings and shows in the next gradient.
+// u1, u2: 1 - b1^step, 1 - b2^step.
 __global__ void adam_kernel(float* __restrict__ params, const float* __restrict__ grads, float* __restrict__ m,
-                            float* __restrict__ v, int n, int step, float lr_rot, float lr_trans, float b1, float b2,
-                            float eps) {
+                            float* __restrict__ v, int n, double u1, double u2, float lr_rot, float lr_trans, float b1,
+                            float b2, float eps) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const float g = grads[i];
-  const float mi = b1 * m[i] + (1.f - b1) * g;
-  const float vi = b2 * v[i] + (1.f - b2) * g * g;
-  m[i] = mi;
-  v[i] = vi;
-  const float mh = mi / (1.f - powf(b1, static_cast<float>(step)));
-  const float vh = vi / (1.f - powf(b2, static_cast<float>(step)));
-  const float lr = (i % 6) < 3 ? lr_rot : lr_trans;
-  params[i] -= lr * mh / (sqrtf(vh) + eps);
+  const double g = grads[i], d1 = b1, d2 = b2;
+  const double mi = fma(d1, static_cast<double>(m[i]), (1.0 - d1) * g);
+  const double vi = fma(d2, static_cast<double>(v[i]), (1.0 - d2) * g * g);
+  m[i] = static_cast<float>(mi);
+  v[i] = static_cast<float>(vi);
+  const double lr = (i % 6) < 3 ? lr_rot : lr_trans;
+  params[i] = static_cast<float>(params[i] - lr * (mi / u1) / (sqrt(vi / u2) + static_cast<double>(eps)));
 }
 
 }  // namespace
@@ -278,7 +280,8 @@ extern "C" drr_status drr_adam_step(float* params_dev, const float* grads_dev, f
   if (drr_status s = drr::device_view(v_dev, dev, true, "v", &v_dev)) return s;
   const int n = 6 * B;
   adam_kernel<<<(n + 255) / 256, 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-      params_dev, grads_dev, m_dev, v_dev, n, step, lr_rot, lr_trans, beta1, beta2, eps);
+      params_dev, grads_dev, m_dev, v_dev, n, 1.0 - std::pow(static_cast<double>(beta1), step),
+      1.0 - std::pow(static_cast<double>(beta2), step), lr_rot, lr_trans, beta1, beta2, eps);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return drr::cuda_error(e, "adam launch");
   drr::count_launches(1);

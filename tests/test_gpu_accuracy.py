@@ -67,3 +67,22 @@ def test_stored_jacobian_gradient_stays_infinite(drr, bad):
     G = drr.render_backward(vol, inputs.Detector(100.0, H, W, 1.0, 1.0), torch.zeros((1, 6), device="cuda"),
                             torch.from_numpy(g).cuda(), jac=torch.from_numpy(J).cuda())
     np.testing.assert_array_equal(G.cpu().numpy(), np.full((1, 6), bad, np.float32))
+
+
+def test_adam_moves_the_pose_by_the_fp64_step(drr):
+    # FP32 states, the step between them in FP64: each is the FP64 result rounded once
+    rng = np.random.default_rng(9)
+    B, lr = 500, np.array([0.01] * 3 + [1.0] * 3, np.float32).astype(np.float64)
+    b1, b2, eps = (float(np.float32(x)) for x in (0.9, 0.999, 1e-8))
+    p = rng.uniform(-30, 30, (B, 6)).astype(np.float32)
+    P = torch.from_numpy(p.copy()).cuda()
+    M, V = torch.zeros_like(P), torch.zeros_like(P)
+    for t in (1, 2, 3):
+        g = (rng.normal(size=(B, 6)) * 10.0 ** rng.uniform(-6, 0, (B, 6))).astype(np.float32)
+        m, v, q = (x.cpu().numpy().astype(np.float64) for x in (M, V, P))
+        drr.adam_step(P, torch.from_numpy(g).cuda(), M, V, t, 0.01, 1.0)
+        g = g.astype(np.float64)
+        m, v = b1 * m + (1 - b1) * g, b2 * v + (1 - b2) * g * g
+        q = q - lr * (m / (1 - b1**t)) / (np.sqrt(v / (1 - b2**t)) + eps)
+        for x, ref in ((M, m), (V, v), (P, q)):
+            np.testing.assert_array_equal(x.cpu().numpy(), ref.astype(np.float32))
