@@ -634,8 +634,8 @@ struct SlabRay {
   u64 lX, ldX;     // slot 1's crossing 0: q_2 and q_0 (both + t1) and their steps
   u64 lY, ldY;
   u32 t0, t1;      // rounding bounds (and biases) of the minor loops' coordinates
-  float w1;        // 1 - q_2 at the entry: the first slab's share inside the ray
-  float rest;      // share of the last slab beyond the exit
+  float w1;        // 1 - q_2 at the entry: the first slab's share inside the ray (a ray inside one slab: its length)
+  float rest;      // share of the last slab beyond the exit (0 then)
   bool exact;      // to be summed by exact_rays
   // the forward walk only
   u64 qx;          // q_2 at the exit
@@ -987,9 +987,12 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
   s.ldY = ff_fix(r21.x < 65536.f ? r01 : make_float2(0.f, 0.f));
   s.Y = static_cast<u64>(E[0]) + (s.dy - __umulhi(E[2], s.dy));
   s.Z = static_cast<u64>(E[1]) + (s.dz - __umulhi(E[2], s.dz));
-  s.mX = E[2] + (s.mdX - mul_frac(E[0], s.mdX)) + s.t0;
+  // a ray inside one slab is measured from its entry, as the forward walk's
+  const bool inside = s.cnt[2] == 0;
+  const u64 from = inside ? 0ull : static_cast<u64>(E[2]);
+  s.mX = from + (s.mdX - mul_frac(E[0], s.mdX)) + s.t0;
   s.mZ = static_cast<u64>(E[1]) + (s.mdz - __umulhi(E[0], s.mdz)) + s.t0;
-  s.lX = E[2] + (s.ldX - mul_frac(E[1], s.ldX)) + s.t1;
+  s.lX = from + (s.ldX - mul_frac(E[1], s.ldX)) + s.t1;
   s.lY = E[0] + (s.ldY - mul_frac(E[1], s.ldY)) + s.t1;
   if (s.cnt[2] > 0) {
     // no minor plane beyond the exit is counted at the last dominant crossing:
@@ -1000,7 +1003,8 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
     const u64 ez = s.Z + m * s.dz, lz = static_cast<u64>(s.cnt[1] + 1) << 32;
     if (ez >= lz) s.Z -= min(s.Z, ez - lz + 1ull);
   }
-  s.w1 = E[2] == 0u ? 1.f : static_cast<float>(0u - E[2]) * kTwoM32;
+  s.w1 = inside ? fix_float(len) : (E[2] == 0u ? 1.f : static_cast<float>(0u - E[2]) * kTwoM32);
+  if (inside) s.rest = 0.f;
   if constexpr (!kFwdOnly) {
     if (MODE == kGeoGrad) {
       park->v[kPkE][t] = (1.f - 2.f * amin.x) - 2.f * amin.y;
@@ -1530,12 +1534,14 @@ __device__ __forceinline__ void slab_finish(const VolumeDev& vd, const PoseGeom&
   const int t = threadIdx.x;
   const float v1 = gather<DT>(vd, s.off);
   const float vl = gather<DT>(vd, s.off + s.cnt[0] * s.step[0] + s.cnt[1] * s.step[1] + s.cnt[2] * s.step[2]);
-  // sum w (1 - f), f the unbiased fraction
+  // sum w (1 - f), f the unbiased fraction; inside one slab, sum w (length - f) (its
+  // 1 - f and rest would be two numbers near a slab that cancel to the length)
+  const float to = s.cnt[2] == 0 ? s.w1 : 1.f;
   const float g0 = T.minor[0].x, g1 = T.minor[1].x;
   const float b0 = static_cast<float>(s.t0) * kTwoM32, b1 = static_cast<float>(s.t1) * kTwoM32;
   Sum2 sum = T.S;
-  sum.add(fmaf(-kTwoM32, T.minor[0].y, fmaf(b0, g0, g0)));
-  sum.add(fmaf(-kTwoM32, T.minor[1].y, fmaf(b1, g1, g1)));
+  sum.add(fmaf(-kTwoM32, T.minor[0].y, fmaf(b0, g0, to * g0)));
+  sum.add(fmaf(-kTwoM32, T.minor[1].y, fmaf(b1, g1, to * g1)));
   sum.add_product(v1, s.w1);
   sum.add_product(-s.rest, vl);
   const float F = sum.value();

@@ -6,7 +6,7 @@ import pytest
 
 import oracle
 from paper_2208_12737_gb300 import inputs
-from tests._parity import odet, ovol
+from tests._parity import FP32_TOL, GRAD_TOL, odet, ovol, rel_err
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -86,3 +86,21 @@ def test_adam_moves_the_pose_by_the_fp64_step(drr):
         q = q - lr * (m / (1 - b1**t)) / (np.sqrt(v / (1 - b2**t)) + eps)
         for x, ref in ((M, m), (V, v), (P, q)):
             np.testing.assert_array_equal(x.cpu().numpy(), ref.astype(np.float32))
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1), (3, 3, 3), (2, 4, 31)])
+def test_jacobian_renders_of_grazing_rays(drr, shape):
+    # a detector fine enough for rays that clip an edge inside one slab: their lengths are a
+    # small part of a slab, and are held to the per-pixel tolerance all the same
+    rng = np.random.default_rng(31)
+    vol_np, sp = rng.uniform(0.01, 0.05, shape).astype(np.float32), (1.0, 1.1, 0.9)
+    ext = max(n * s for n, s in zip(shape[::-1], sp))
+    det = inputs.Detector(510.0, 601, 597, 3.6 * ext / 600, 3.6 * ext / 600)
+    poses = inputs.random_poses(4, seed=32, max_angle_deg=40, max_trans_mm=0.3)
+    ov = ovol(vol_np, sp)
+    ref, J_ref = oracle.render(ov, odet(det), poses, jacobian=True)
+    E, J = drr.render(drr.Volume(vol_np, sp), det, torch.from_numpy(poses).cuda(), jacobian=True)
+    assert (ref > 0).sum() > 10000 and rel_err(E.cpu().numpy(), ref).max() < FP32_TOL
+    J, J_ref = J.cpu().numpy(), np.moveaxis(J_ref, -1, 1)
+    for grp in (slice(0, 3), slice(3, 6)):
+        assert (np.abs(J[:, grp] - J_ref[:, grp]) / np.abs(J_ref[:, grp]).max()).max() < GRAD_TOL
