@@ -2281,33 +2281,32 @@ __device__ __forceinline__ void sum_pose_partials(const float* __restrict__ p, i
                                                   float* __restrict__ out) {
   __shared__ double wsum[kFinThreads / 32][6];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  float2 s[6];
-#pragma unroll
-  for (int k = 0; k < 6; ++k) s[k] = make_float2(0.f, 0.f);
+  Sum2 s[6];
 #pragma unroll 4
   for (int c = t; c < nt; c += kFinThreads) {
     const float* row = p + static_cast<size_t>(c) * ncol;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      if (k < ncol) {
-        const float2 x = ff_sum(s[k].x, row[k]);
-        s[k] = make_float2(x.x, __fadd_rn(s[k].y, x.y));
-      }
-    }
+    for (int k = 0; k < 6; ++k)
+      if (k < ncol) s[k].add(row[k]);
   }
+  bool finite = true;
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
+    s[k].warp_sum();
+    finite = finite && isfinite(s[k].s);
+    if (lane == 0) wsum[warp][k] = s[k].value64();
+  }
+  if (__syncthreads_or(!finite)) {  // infinite partial sums, or sums beyond FP32's range: again in FP64
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float2 x = ff_sum(s[k].x, __shfl_xor_sync(0xffffffffu, s[k].x, o));
-      s[k] = make_float2(x.x, __fadd_rn(__fadd_rn(s[k].y, __shfl_xor_sync(0xffffffffu, s[k].y, o)), x.y));
+    for (int k = 0; k < 6; ++k) {
+      double x = 0.0;
+      for (int c = t; k < ncol && c < nt; c += kFinThreads) x += static_cast<double>(p[static_cast<size_t>(c) * ncol + k]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      if (lane == 0) wsum[warp][k] = x;
     }
+    __syncthreads();
   }
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) wsum[warp][k] = static_cast<double>(s[k].x) + static_cast<double>(s[k].y);
-  }
-  __syncthreads();
   if (t < ncol) {
     double a = 0.0;
 #pragma unroll

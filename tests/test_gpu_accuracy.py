@@ -104,3 +104,36 @@ def test_jacobian_renders_of_grazing_rays(drr, shape):
     J, J_ref = J.cpu().numpy(), np.moveaxis(J_ref, -1, 1)
     for grp in (slice(0, 3), slice(3, 6)):
         assert (np.abs(J[:, grp] - J_ref[:, grp]) / np.abs(J_ref[:, grp]).max()).max() < GRAD_TOL
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf])
+def test_gradient_sums_stay_infinite(drr, bad):
+    # one infinite upstream gradient, without a stored Jacobian and with one, pose and detector parameters
+    vol = drr.Volume(np.random.default_rng(33).uniform(0.01, 0.05, (20, 22, 24)).astype(np.float32), (1.0, 1.1, 0.9))
+    det = inputs.Detector(150.0, 45, 37, 0.8, 0.8)
+    P = torch.from_numpy(inputs.random_poses(2, seed=34)).cuda()
+    E, J = drr.render(vol, det, P, jacobian=True)
+    g = torch.ones_like(E)
+    h, w = (int(x) for x in torch.nonzero((J[1] != 0).all(0))[50])
+    g[1, h, w] = bad
+    G = drr.render_backward(vol, det, P, g).cpu().numpy()
+    np.testing.assert_array_equal(G[1], bad * np.sign(J[1, :, h, w].cpu().numpy()))
+    np.testing.assert_array_equal(G[1], drr.render_backward(vol, det, P, g, jac=J).cpu().numpy()[1])
+    assert np.isfinite(G[0]).all()
+    assert np.isinf(drr.geometry_grad(vol, det, P, g).cpu().numpy()[1]).all()
+
+
+def test_gradient_sums_beyond_fp32_that_cancel(drr):
+    # rows of tiles of opposite signs, each tile's sum just within FP32: 32 of one sign are not
+    vol = drr.Volume(np.full((20, 60, 60), 0.03, np.float32), (3.0, 1.0, 1.0))
+    det = inputs.Detector(200.0, 16, 512, 1.0, 0.1)
+    P = torch.from_numpy(np.array([[0.02, 0.03, 0.01, 1.0, 0.5, 0.3]], np.float32)).cuda()
+    E, J = drr.render(vol, det, P, jacobian=True)
+    J = J[0].cpu().numpy().astype(np.float64)
+    tiles = np.abs(J).reshape(6, 4, 4, 64, 8).sum((2, 4))
+    sign = np.repeat([1.0, -1.0, -1.0, 1.0], 4)[:, None]
+    g = (np.broadcast_to(sign, (16, 512)) * (2.5e38 / tiles[0].max())).astype(np.float32)  # (rz's tiles; ry's overflow)
+    ref, terms = (J * g).sum((1, 2)), np.abs(J * g).sum((1, 2))
+    G = drr.render_backward(vol, det, P, torch.from_numpy(g[None].copy()).cuda()).cpu().numpy()[0].astype(np.float64)
+    assert terms[0] > 8 * 2 * 3.4e38 and abs(ref[0]) < 3e38  # eight warps of 32 tiles each
+    assert abs(G[0] - ref[0]) <= 1e-5 * terms[0]  # (1e-5: what the two walks' Jacobians may differ by)
