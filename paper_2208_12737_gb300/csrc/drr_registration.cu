@@ -17,16 +17,19 @@ namespace {
 // One thread-block cluster per image pair; block r takes the r-th contiguous
 // share of the pixels.  What bounded one block per pair was FP64 arithmetic (15
 // operations per pixel at 1/64 of the FP32 rate), on one SM per pair.  Per thread
-// the sums now run in FP32 with exact products and exact sums (value + error,
-// Knuth / Dekker), ~2^-47 of a partial sum, and only the threads' partial sums
-// are added in FP64; the image gradient is evaluated the same way from FP64
-// coefficients.  Measured (call with gradient, CUDA events): one 256x256 pair
-// 306 -> 19 us, 64 pairs 308 -> 31 us, 8 pairs of 1024x1024 4400 -> 150 us; 256
-// pairs of 200x200 without gradient 212 -> 68 us, 4096 of them 2770 -> 961 us (two
+// the sums now run in FP32 with exact products, kept as value + error (Knuth /
+// Dekker), and only the threads' partial sums are added in FP64; the image gradient
+// is evaluated the same way from FP64 coefficients.  The errors are added in FP32:
+// a sum of 2^20 pixels is good to ~2^-43, and a variance to as much of the mean
+// square.  Images whose mean square is above kZWide variances (where that would reach
+// FP32's bits: 1.7e-5 at a mean of 10^4 deviations) are taken in FP64.  Measured (call with gradient, CUDA events): one 256x256 pair
+// 306 -> 19 us, 64 pairs 308 -> 29 us, 8 pairs of 1024x1024 4400 -> 150 us; 256
+// pairs of 200x200 without gradient 212 -> 64 us, 4096 of them 2770 -> 907 us (two
 // thirds of that the FP64 sums of the partial sums and the closing scalars).
 constexpr int kZThreads = 256;
 constexpr int kZCluster = 8;  // the portable cluster size
 constexpr int kZSums = 5;     // sum I, I^2, F, F^2, I F
+constexpr double kZWide = 128.0;
 
 struct Acc {  // s + e, an unevaluated sum
   float s = 0.f, e = 0.f;
@@ -96,9 +99,10 @@ __global__ void __cluster_dims__(kZCluster, 1, 1) __launch_bounds__(kZThreads)
   // every block says so here, and the first remote write below waits for all
   cluster.barrier_arrive();
   __shared__ double part[kZSums][kZThreads];
-  __shared__ float range[kZThreads / 32];
-  __shared__ double rows[kZCluster][kZSums + 1];  // every block's sums and largest magnitude
+  __shared__ float range[2][kZThreads / 32];
+  __shared__ double rows[kZCluster][kZSums + 2];  // every block's sums and largest magnitudes (I, F)
   __shared__ Coefficients coef;
+  __shared__ int again;
   __shared__ double coef64[3];
   const float* I = moving + static_cast<size_t>(pair) * npix;
   const float* F = fixed + static_cast<size_t>(pair) * fixed_stride;
@@ -108,11 +112,11 @@ __global__ void __cluster_dims__(kZCluster, 1, 1) __launch_bounds__(kZThreads)
   // products and coefficients of images far from 1 in magnitude would leave the
   // range of FP32: such images (and images that are not finite) are taken in FP64
   int wide = 0;
+  double v[kZSums];  // the pair's sums (thread 0)
   for (;; ++wide) {
-    float largest = 0.f;
+    float mi = 0.f, mf = 0.f;
     if (!wide) {
       Acc s[kZSums];
-      float mi = 0.f, mf = 0.f;
       each_pixel(I, F, lo, hi, vec, [&](int, float a, float b) {
         s[0].add(a);
         s[1].add_product(a, a);
@@ -122,14 +126,13 @@ __global__ void __cluster_dims__(kZCluster, 1, 1) __launch_bounds__(kZThreads)
         mi = fmaxf(mi, fabsf(a));
         mf = fmaxf(mf, fabsf(b));
       });
-      const auto fits = [](float m) { return m == 0.f || (m > 1e-8f && m < 1e10f); };
-      bool ok = true;
 #pragma unroll
       for (int k = 0; k < kZSums; ++k) {
         part[k][t] = static_cast<double>(s[k].s) + static_cast<double>(s[k].e);
-        ok = ok && isfinite(s[k].s) && isfinite(s[k].e);
+        if (!isfinite(s[k].s) || !isfinite(s[k].e)) mi = __int_as_float(0x7f800000);
       }
-      largest = ok && fits(mi) && fits(mf) ? 0.f : 1.f;
+      const auto in_range = [](float m) { return m == 0.f || (m > 1e-8f && m < 1e10f); };
+      if (!in_range(mi) || !in_range(mf)) mi = __int_as_float(0x7f800000);
     } else {
       double s[kZSums] = {0.0, 0.0, 0.0, 0.0, 0.0};
       each_pixel(I, F, lo, hi, vec, [&](int, float x, float y) {
@@ -143,8 +146,13 @@ __global__ void __cluster_dims__(kZCluster, 1, 1) __launch_bounds__(kZThreads)
 #pragma unroll
       for (int k = 0; k < kZSums; ++k) part[k][t] = s[k];
     }
-    const bool any = __any_sync(0xffffffffu, largest != 0.f);
-    if (lane == 0) range[warp] = any ? 1.f : 0.f;
+    // (the bits of numbers that are not negative are in the numbers' order)
+    const unsigned int ri = __reduce_max_sync(0xffffffffu, __float_as_uint(mi)),
+                       rf = __reduce_max_sync(0xffffffffu, __float_as_uint(mf));
+    if (lane == 0) {
+      range[0][warp] = __uint_as_float(ri);
+      range[1][warp] = __uint_as_float(rf);
+    }
     __syncthreads();
     if (!wide) cluster.barrier_wait();  // (the second pass: the sync at the end of the first)
     if (warp < kZSums) {  // warp k: the block's sum k, in a fixed order
@@ -154,29 +162,41 @@ __global__ void __cluster_dims__(kZCluster, 1, 1) __launch_bounds__(kZThreads)
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
       // to every block of the cluster (one of its lanes each)
-      if (lane < kZCluster) cluster.map_shared_rank(&rows[0][0], lane)[rank * (kZSums + 1) + warp] = x;
-    } else if (warp == kZSums && lane < kZCluster) {
-      double x = 0.0;
+      if (lane < kZCluster) cluster.map_shared_rank(&rows[0][0], lane)[rank * (kZSums + 2) + warp] = x;
+    } else if (warp < kZSums + 2 && lane < kZCluster) {
+      float x = 0.f;
 #pragma unroll
-      for (int q = 0; q < kZThreads / 32; ++q) x = fmax(x, static_cast<double>(range[q]));
-      cluster.map_shared_rank(&rows[0][0], lane)[rank * (kZSums + 1) + kZSums] = x;
+      for (int q = 0; q < kZThreads / 32; ++q) x = fmaxf(x, range[warp - kZSums][q]);
+      cluster.map_shared_rank(&rows[0][0], lane)[rank * (kZSums + 2) + warp] = static_cast<double>(x);
     }
     cluster.sync();  // every block's rows are complete in every block
-    bool again = false;
+    if (t == 0) {    // the same in every block
 #pragma unroll
-    for (int r = 0; r < kZCluster; ++r) again = again || rows[r][kZSums] != 0.0;
+      for (int k = 0; k < kZSums; ++k) {
+        double x = 0.0;
+#pragma unroll
+        for (int r = 0; r < kZCluster; ++r) x += rows[r][k];
+        v[k] = x;
+      }
+      double li = 0.0, lf = 0.0;  // the images' largest magnitudes
+#pragma unroll
+      for (int r = 0; r < kZCluster; ++r) {
+        li = fmax(li, rows[r][kZSums]);
+        lf = fmax(lf, rows[r][kZSums + 1]);
+      }
+      const auto fits = [](double m) { return m == 0.0 || (m > 1e-8 && m < 1e10); };
+      // mean square x^2 <= kZWide (x^2 - mean^2), with n = npix: q n <= kZWide (q n - m m)
+      const auto spread = [&](double m, double q) {
+        const double qn = q * static_cast<double>(npix);
+        return qn <= kZWide * (qn - m * m);
+      };
+      again = !(fits(li) && fits(lf) && spread(v[0], v[1]) && spread(v[2], v[3]));
+    }
+    __syncthreads();
     if (wide || !again) break;
     cluster.sync();  // all blocks have read the rows before they are written again
   }
   if (t == 0 && (grad || rank == 0)) {  // every block needs the coefficients, one the loss
-    double v[kZSums];
-#pragma unroll
-    for (int k = 0; k < kZSums; ++k) {
-      double x = 0.0;
-#pragma unroll
-      for (int r = 0; r < kZCluster; ++r) x += rows[r][k];
-      v[k] = x;
-    }
     const double inv = 1.0 / static_cast<double>(npix);
     const double mi = v[0] * inv, mf = v[2] * inv;
     const double si = sqrt(fmax(v[1] * inv - mi * mi, 0.0)), sf = sqrt(fmax(v[3] * inv - mf * mf, 0.0));
