@@ -131,8 +131,6 @@ __global__ void __cluster_dims__(kZCluster, 1, 1) __launch_bounds__(kZThreads)
         part[k][t] = static_cast<double>(s[k].s) + static_cast<double>(s[k].e);
         if (!isfinite(s[k].s) || !isfinite(s[k].e)) mi = __int_as_float(0x7f800000);
       }
-      const auto in_range = [](float m) { return m == 0.f || (m > 1e-8f && m < 1e10f); };
-      if (!in_range(mi) || !in_range(mf)) mi = __int_as_float(0x7f800000);
     } else {
       double s[kZSums] = {0.0, 0.0, 0.0, 0.0, 0.0};
       each_pixel(I, F, lo, hi, vec, [&](int, float x, float y) {

@@ -35,3 +35,27 @@ def test_correlated_images_far_from_zero(drr, shape, mean):
     assert np.abs(loss.cpu().numpy() - ref).max() < tol + 2.0**-24
     scale = np.abs(g_ref).max()
     assert np.abs(g.cpu().numpy() - g_ref).max() < (4 * tol + 2.0**-22) * scale
+
+
+def test_one_small_pixel_does_not_change_the_path(drr):
+    # (a ray that clips a corner): once sent the pair through a second pass, in FP64
+    rng = np.random.default_rng(52)
+    I = torch.from_numpy(rng.uniform(0, 5, (32, 1024, 1024)).astype(np.float32)).cuda()
+    F = (0.5 * I + 1.0).contiguous()
+    J = I.clone()
+    J[:, :, :4] = 0.0  # (all pixels of some threads)
+    J[:, 0, 0] = 1e-12
+
+    def ms(A):
+        best = np.inf
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            drr.zncc(A, F, grad=False)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+
+    plain, odd = ms(I), ms(J)
+    assert odd < 1.5 * plain, (odd, plain)
