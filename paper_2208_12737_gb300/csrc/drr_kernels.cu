@@ -48,7 +48,8 @@ struct Voxel<kF16> {
 
 // Bounds-checked build (-DDRR_CHECK_BOUNDS=1, a separate library built for
 // tests): every voxel gather is checked against the padded volume and every
-// back-projection add of a live segment against the gradient volume; a check
+// back-projection add of a live segment against the gradient volume, but for
+// segments shorter than the rounding of their ends (walk_backproject); a check
 // that fails sets a bit of a device-wide fault word (read and cleared by
 // drr_stream_check, which then returns DRR_ERR_DEVICE) and skips the access.
 // The product build has no checks: the zero padding keeps every gather of the
@@ -1973,8 +1974,12 @@ __device__ __forceinline__ void walk_backproject(const VolumeDev& vd, const Slab
       const float end = fminf(fmaxf(an, lo), xe);
       const bool on = static_cast<u32>(live) < static_cast<u32>(nseg);
 #if DRR_CHECK_BOUNDS
-      // crossings closer than FP32 resolves may come in another order at the exit: a segment of no length
-      if (on && at >= nvox && end - ac > 1e-4f) atomicOr(&g_fault_word, kFaultBackproject);
+      // Crossings closer than the positions' rounding may come in another order at the exit, with a
+      // segment beyond it that is dropped: two positions l r + x0 (three roundings each, 2^-23 of the
+      // position in all) apart by less, and the fixed-point ends by their own 2^-32 of a plane.
+      const float tie = fmaf(2.384185791015625e-7f, fmaxf(fabsf(end), fabsf(ac)),
+                             fmaf(9.313225746154785e-10f, s.r0 + s.r1, 5.9604644775390625e-8f));  // 2^-22, 2^-30, 2^-24
+      if (on && at >= nvox && end - ac > tie) atomicOr(&g_fault_word, kFaultBackproject);
 #endif
       red_column_merged<kBpTileW>(gvol, on ? at : 0xffffffffu, gL * (end - ac), nvox, lane);
       ac = end;
