@@ -143,8 +143,8 @@ cudaError_t launch_plain_fd_finish(const float* E13, int B, int npix, float h_ro
 cudaError_t launch_zncc(const float* moving, const float* fixed, size_t fixed_stride, int B, int npix, float eps,
                         float* loss, float* grad, cudaStream_t stream);
 // Pose gradient by re-tracing: one partial sum of g . J per warp tile
-// (partials: B * pose_tiles(det) * 6 floats), then the fixed-order FP64
-// finalize over nblk = pose_tiles(det) partials per pose.
+// (partials: B * pose_tiles(det) * 6 floats), then the fixed-order finalize (value +
+// error pairs, to FP64 accuracy) over nblk = pose_tiles(det) partials per pose.
 cudaError_t launch_pose_grad_walk(const VolumeDev& vd, const DetDev& det, const PoseGeom* pg, int B,
                                   const float* grad_drr, float* partials, cudaStream_t stream);
 cudaError_t launch_pose_grad_finalize(const float* partials, int B, int nblk, float* grad_pose, cudaStream_t stream);

@@ -283,14 +283,16 @@ __global__ void ray_setup_kernel(const float* __restrict__ poses, int B, DetDev 
 }
 
 // ---------------------------------------------------------------------------
-// One ray: FP64 clip and entry (Sec. 2.3), then the FP32 incremental walk.
+// One ray: the FP64 clip and entry (Sec. 2.3) of the rays that slab_setup cannot
+// decide, and of the segment count.
 // ---------------------------------------------------------------------------
 struct RayResult {
-  float F;     // E (or the raw sum in alpha units before the final scaling)
+  float F;     // E
   float J[6];  // dE/d eta (only for the Jacobian modes)
 };
 
-// Per-ray state after the FP64 setup: everything the walk needs.
+// Per-ray state after the FP64 setup, for exact_rays, backproject_exact and the
+// segment count (mode kCount).
 //
 // Crossing parameters are fixed point: alpha measured from the entry is held
 // as a 32.32 number in units of span / 2^24 (span = alpha_max - alpha_min), so
@@ -547,17 +549,18 @@ __device__ __forceinline__ float local_pos(unsigned long long x, unsigned long l
 // w times its position are those of the two minor loops; the dominant axis'
 // follow from sum w = 0 and sum w alpha = F over all crossings.
 // Measured (fused forward + Jacobian kernel, FP32, CUDA events): 16-pose CT
-// batch, 512x512x133 and 200x200, 0.559 -> 0.413 ms against the walk that merged
-// the axes' crossings in order (429 -> 267 M warp instructions); 150x141 on 256^3
-// split over the warps of a tile, 0.067 -> 0.051 ms.  What bounds it now is the L1
-// data pipe (82 % busy): the dominant loop's gathers touch ~15 lines each (rays of
+// batch, 512x512x133 and 200x200, 0.559 -> 0.427 ms against the walk that merged
+// the axes' crossings in order (429 -> 273 M warp instructions); 150x141 on 256^3
+// split over the warps of a tile, 0.067 -> 0.042 ms.  What bounds it now is the L1
+// data pipe (78 % busy): the dominant loop's gathers touch ~15 lines each (rays of
 // a tile at one plane x = const of an x-fastest volume), ~5 wavefronts.  Taking
 // 2 x 4 rays and 4 planes per gather (35 instead of 50 M wavefronts but more L2
 // sectors, 0.469 ms), the three loops interleaved in chunks (0.505), and a second
 // copy of the volume with another fastest axis (17 M wavefronts, but every
 // gather an L2 access and 0.74 GB from DRAM: 0.446) were slower.  The forward
 // alone keeps the merged walk: it gathers once per segment, the slab walk once
-// per slab and twice per minor crossing (0.391 against 0.366 ms).
+// per slab and twice per minor crossing (0.391 ms when the merged one took 0.366; it
+// takes 0.344 now).
 //
 // Coordinates run in the ray's direction on every axis, from the entry voxel's
 // lower plane: q_a in [0, 1] at the entry, crossing k of axis a at q_a = 1 + k.
@@ -574,6 +577,11 @@ __device__ __forceinline__ float local_pos(unsigned long long x, unsigned long l
 // at a time), and the pieces' sums are added in order: the split kernel, whose
 // warps take different pieces, gives the same bits.
 // ---------------------------------------------------------------------------
+// Measured (us; lone 150x141 on 256^3, CT batch, 4 poses of 509x451 on 512x512x300 BF16):
+// pieces of 32 planes, 8 of them, 8 slabs and 4 minor crossings in flight 42 / 428 / 618;
+// pieces of 16 or 64 the same; 4 pieces 43 / 426 / 605, but twice as many planes to look
+// through for a pair (settle_pairs) and half the warps of a split tile idle; 4 slabs in
+// flight 42 / 464 / 655, 16 41 / 421 / 622; 2 minor crossings 43 / 454 / 678, 8 43 / 443 / 647.
 #ifndef DRR_PIECE_LEN
 #define DRR_PIECE_LEN 32
 #endif
@@ -1041,7 +1049,7 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
 // of a ray, give the same bits as one warp walking through.
 //
 // What bounds it: one gather per segment, 4.4 wavefronts each on the L1 data
-// pipe (71 % busy), and ~18 warp instructions per segment (issue slots 60 %).
+// pipe (68 % busy), and ~18 warp instructions per segment (issue slots 61 %).
 // Measured (CUDA events): 16-pose CT batch, 512x512x133 and 200x200, 0.366 ->
 // 0.344 ms against the walk with an FP64 ray setup; one 128x128 pose on 256^3, split
 // over the warps of a tile, 0.069 -> 0.028.  Chunks that begin at a dominant

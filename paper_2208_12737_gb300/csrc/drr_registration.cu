@@ -22,10 +22,11 @@ namespace {
 // is evaluated the same way from FP64 coefficients.  The errors are added in FP32:
 // a sum of 2^20 pixels is good to ~2^-43, and a variance to as much of the mean
 // square.  Images whose mean square is above kZWide variances (where that would reach
-// FP32's bits: 1.7e-5 at a mean of 10^4 deviations) are taken in FP64.  Measured (call with gradient, CUDA events): one 256x256 pair
-// 306 -> 19 us, 64 pairs 308 -> 29 us, 8 pairs of 1024x1024 4400 -> 150 us; 256
-// pairs of 200x200 without gradient 212 -> 64 us, 4096 of them 2770 -> 907 us (two
-// thirds of that the FP64 sums of the partial sums and the closing scalars).
+// FP32's bits: 1.7e-5 at a mean of 10^4 deviations) are taken in FP64.  Measured
+// (call with gradient, CUDA events): one 256x256 pair 306 -> 19 us, 64 pairs 308 -> 29
+// us, 8 pairs of 1024x1024 4400 -> 146 us; 256 pairs of 200x200 without gradient 212 ->
+// 64 us, 4096 of them 2770 -> 907 us (two thirds of that the FP64 sums of the partial
+// sums and the closing scalars).
 constexpr int kZThreads = 256;
 constexpr int kZCluster = 8;  // the portable cluster size
 constexpr int kZSums = 5;     // sum I, I^2, F, F^2, I F
