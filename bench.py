@@ -999,8 +999,9 @@ def run_ours(args, rank, world, local_rank):
         # Gather roofline: voxel bytes gathered per second by the dominant kernel (segments x
         # element size / its event-timed launch) against the measured HBM copy bandwidth, and
         # beside it against the L2 read bandwidth probed in this run.  What binds the kernel is
-        # instruction issue (`issue`: ncu warp instructions per launch / launch time / the issue
-        # peak of 4 schedulers x SMs x max clock); the gathers stay well below both ceilings.
+        # the L1 data pipe (~5 wavefronts per 32-lane gather, 79 % busy in profiles/); `issue`: ncu
+        # warp instructions per launch / launch time / the issue peak of 4 schedulers x SMs x max
+        # clock.  The gathers stay well below both ceilings.
         "roofline": {"bound": "hbm", "achieved": gather_gbs, "peak": hbm, "unit": "GB/s",
                      "frac": gather_gbs / hbm, "traffic": profiled_traffic("siddon_fwd_jac"),
                      "kernel": "siddon_fwd_jac", "kernel_ms": k_ms,
@@ -1010,7 +1011,7 @@ def run_ours(args, rank, world, local_rank):
                      "l2": {"achieved_gbs": gather_gbs, "peak_gbs": l2, "frac": gather_gbs / l2,
                             "peak_source": "measured in this run: 64 MB L2-resident buffer streamed with "
                                            "16-byte L2-only loads (drr_probe_l2_read)"},
-                     "limiter": "issue",
+                     "limiter": "l1_data_pipe",
                      "issue": issue,
                      # aside: a hand-counted 8 essential FP32 ops per segment against the FP32 lanes
                      "alu_aside": {"ops_per_segment": ops_per_seg,

@@ -550,9 +550,9 @@ __device__ __forceinline__ float local_pos(unsigned long long x, unsigned long l
 // follow from sum w = 0 and sum w alpha = F over all crossings.
 // Measured (fused forward + Jacobian kernel, FP32, CUDA events): 16-pose CT
 // batch, 512x512x133 and 200x200, 0.559 -> 0.427 ms against the walk that merged
-// the axes' crossings in order (429 -> 273 M warp instructions); 150x141 on 256^3
+// the axes' crossings in order (429 -> 269 M warp instructions); 150x141 on 256^3
 // split over the warps of a tile, 0.067 -> 0.042 ms.  What bounds it now is the L1
-// data pipe (78 % busy): the dominant loop's gathers touch ~15 lines each (rays of
+// data pipe (79 % busy): the dominant loop's gathers touch ~15 lines each (rays of
 // a tile at one plane x = const of an x-fastest volume), ~5 wavefronts.  Taking
 // 2 x 4 rays and 4 planes per gather (35 instead of 50 M wavefronts but more L2
 // sectors, 0.469 ms), the three loops interleaved in chunks (0.505), and a second
@@ -1049,7 +1049,7 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
 // of a ray, give the same bits as one warp walking through.
 //
 // What bounds it: one gather per segment, 4.4 wavefronts each on the L1 data
-// pipe (68 % busy), and ~18 warp instructions per segment (issue slots 61 %).
+// pipe (68 % busy), and ~18 warp instructions per segment (issue slots 62 %).
 // Measured (CUDA events): 16-pose CT batch, 512x512x133 and 200x200, 0.366 ->
 // 0.344 ms against the walk with an FP64 ray setup; one 128x128 pose on 256^3, split
 // over the warps of a tile, 0.069 -> 0.028.  Chunks that begin at a dominant
