@@ -722,14 +722,6 @@ struct Sum2 {
       add(Sum2{__shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, e, o)});
   }
 };
-__device__ __forceinline__ float2 ff_sqr(float2 a) {
-  const float p = __fmul_rn(a.x, a.x);
-  return ff_norm(p, __fmaf_rn(__fadd_rn(a.x, a.x), a.y, __fmaf_rn(a.x, a.x, -p)));
-}
-__device__ __forceinline__ float2 ff_sqrt(float2 a) {  // 1e-30 < a < 1e30
-  const float r = __fsqrt_rn(a.x);
-  return ff_norm(r, __fmul_rn(__fadd_rn(__fmaf_rn(-r, r, a.x), a.y), __fmul_rn(0.5f, __frcp_rn(r))));
-}
 // a times c, rounded once (to its last bit or so).
 __device__ __forceinline__ float ff_scaled(const Sum2& a, float2 c) {
   const float p = __fmul_rn(a.s, c.x);
@@ -1025,9 +1017,20 @@ __device__ __forceinline__ int slab_setup(const VolumeDev& vd, const PoseGeom& p
     park->v[kPkSpan][t] = fix_float(len) * sr[2].x;
     // the path length of a slab as float-float: the roundings of an FP32 product of
     // length and alpha per slab were a third of a pixel's error
-    const auto side = [&](int k) { return make_float2(pick3(ax[k], vd.delta[0], vd.delta[1], vd.delta[2]), 0.f); };
-    const float2 sq = ff_add(ff_add(ff_sqr(ff_mul(r02, side(0))), ff_sqr(ff_mul(r12, side(1)))), ff_sqr(side(2)));
-    const float2 mm = sq.x > 1e-24f && sq.x < 1e30f ? ff_sqrt(sq) : make_float2(L * sr[2].x, 0.f);
+    const auto side = [&](int k) { return pick3(ax[k], vd.delta[0], vd.delta[1], vd.delta[2]); };
+    Sum2 sq;
+    sq.add_product(side(2), side(2));
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float2 r = k == 0 ? r02 : r12;
+      const float x = __fmul_rn(r.x, side(k)), xl = __fmaf_rn(r.y, side(k), __fmaf_rn(r.x, side(k), -x));
+      sq.add_product(x, x);
+      sq.e = __fmaf_rn(__fadd_rn(x, x), xl, sq.e);
+    }
+    const float root = __fsqrt_rn(sq.s);
+    const float2 mm = sq.s > 1e-24f && sq.s < 1e30f
+                          ? make_float2(root, __fadd_rn(__fmaf_rn(-root, root, sq.s), sq.e) * __fdividef(0.5f, root))
+                          : make_float2(L * sr[2].x, 0.f);
     park->v[kPkMm][t] = mm.x;
     park->v[kPkMm + 1][t] = mm.y;
   }
@@ -1391,17 +1394,16 @@ __device__ __forceinline__ void least_loop(const VolumeDev& vd, const SlabRay& s
 #undef DRR_MINOR_PIECES
 #undef DRR_MINOR_BLOCK
 
-// Whole-ray sums of one minor axis' pieces, added in piece order as value + error.
+// Whole-ray sums of one minor axis' pieces, added in piece order.
 struct MinorTotals {
-  Sum2 g, c, h;
+  float g = 0.f, c = 0.f, h = 0.f;
   // first: the piece's first crossing (h counts from the ray's)
   __device__ __forceinline__ void add(float pg, float pc, float ph, int first) {
-    g.add(pg);
-    c.add(pc);
-    h.add(ph);
-    h.add_product(static_cast<float>(first), pg);
+    g += pg;
+    c += pc;
+    h += fmaf(static_cast<float>(first), pg, ph);
   }
-  __device__ __forceinline__ float3 value() const { return make_float3(g.value(), c.value(), h.value()); }
+  __device__ __forceinline__ float3 value() const { return make_float3(g, c, h); }
 };
 struct SlabTotals {
   Sum2 S;
