@@ -999,7 +999,7 @@ def run_ours(args, rank, world, local_rank):
         # Gather roofline: voxel bytes gathered per second by the dominant kernel (segments x
         # element size / its event-timed launch) against the measured HBM copy bandwidth, and
         # beside it against the L2 read bandwidth probed in this run.  What binds the kernel is
-        # the L1 data pipe (~5 wavefronts per 32-lane gather, 79 % busy in profiles/); `issue`: ncu
+        # the L1 data pipe (~5 wavefronts per 32-lane gather, 81 % busy in profiles/); `issue`: ncu
         # warp instructions per launch / launch time / the issue peak of 4 schedulers x SMs x max
         # clock.  The gathers stay well below both ceilings.
         "roofline": {"bound": "hbm", "achieved": gather_gbs, "peak": hbm, "unit": "GB/s",

@@ -549,10 +549,10 @@ __device__ __forceinline__ float local_pos(unsigned long long x, unsigned long l
 // w times its position are those of the two minor loops; the dominant axis'
 // follow from sum w = 0 and sum w alpha = F over all crossings.
 // Measured (fused forward + Jacobian kernel, FP32, CUDA events): 16-pose CT
-// batch, 512x512x133 and 200x200, 0.559 -> 0.427 ms against the walk that merged
-// the axes' crossings in order (429 -> 269 M warp instructions); 150x141 on 256^3
+// batch, 512x512x133 and 200x200, 0.559 -> 0.421 ms against the walk that merged
+// the axes' crossings in order (429 -> 259 M warp instructions); 150x141 on 256^3
 // split over the warps of a tile, 0.067 -> 0.042 ms.  What bounds it now is the L1
-// data pipe (79 % busy): the dominant loop's gathers touch ~15 lines each (rays of
+// data pipe (81 % busy): the dominant loop's gathers touch ~15 lines each (rays of
 // a tile at one plane x = const of an x-fastest volume), ~5 wavefronts.  Taking
 // 2 x 4 rays and 4 planes per gather (35 instead of 50 M wavefronts but more L2
 // sectors, 0.469 ms), the three loops interleaved in chunks (0.505), and a second
@@ -577,7 +577,7 @@ __device__ __forceinline__ float local_pos(unsigned long long x, unsigned long l
 // at a time), and the pieces' sums are added in order: the split kernel, whose
 // warps take different pieces, gives the same bits.
 // ---------------------------------------------------------------------------
-// Measured (us; lone 150x141 on 256^3, CT batch, 4 poses of 509x451 on 512x512x300 BF16):
+// Measured in one run (us; lone 150x141 on 256^3, CT batch, 4 poses of 509x451 on 512x512x300 BF16):
 // pieces of 32 planes, 8 of them, 8 slabs and 4 minor crossings in flight 42 / 428 / 618;
 // pieces of 16 or 64 the same; 4 pieces 43 / 426 / 605, but twice as many planes to look
 // through for a pair (settle_pairs) and half the warps of a split tile idle; 4 slabs in
@@ -1543,10 +1543,10 @@ __device__ __noinline__ void exact_rays(const VolumeDev& vd, const PoseGeom& pg,
 // again, without gathers but for the pairs.  On a generic pose 1 ray in 2000 has a
 // pair, on axis-aligned ones up to half of them do, with ~3 each.  Such rays summed
 // again one after another (exact_rays) took 8 times as long as the walk.  Measured
-// with Jacobian, 16 poses of 256x256 at 1 mm on 256^3: no rotation 3335 -> 660 us, a
-// quarter turn 1937 -> 567, generic poses 397 -> 406; CT batch unrotated 586 -> 350.
-// Of the 660: 300 the walk, 70 the second setup, 95 looking for the pairs.  With FP64
-// positions compared pair by pair 817.
+// with Jacobian, 16 poses of 256x256 at 1 mm on 256^3: no rotation 3335 -> 637 us, a
+// quarter turn 1937 -> 540, generic poses 397 -> 390; CT batch unrotated 586 -> 341.
+// Of the first, 300 are the walk, 70 the second setup, 95 looking for the pairs; with
+// FP64 positions compared pair by pair it took 160 more.
 template <int DT>
 __device__ __forceinline__ void settle_pairs(const VolumeDev& vd, const PoseGeom& pg, int h, int w, const SlabRay& s,
                                              const Plan& pl, u32 near, SlabTotals& T) {
